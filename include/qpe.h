@@ -399,7 +399,7 @@ typedef struct {
  * allocation would synchronise or grow a memory pool that must stay fixed,
  * or a host library that never owns device memory), so it needs no
  * workspace: its only scratch, the per-block partial results, is a fixed
- * array inside the library (256 KiB on every GPU that loads it, held until
+ * array inside the library (24 KiB on every GPU that loads it, held until
  * the process exits).
  *
  * final_state: device pointer to the N x d final statevector in natural row
@@ -408,7 +408,7 @@ typedef struct {
  * (N doubles, P[y] = sum_t |X[y][t]|^2) and *readout. Enqueued on
  * cuda_stream (a cudaStream_t, NULL = legacy default stream); no host
  * synchronisation. Nmeas above 21 is rejected with QPE_ERR_WORKSPACE (the
- * fixed scratch holds 8192 partials of 256 rows each); bad pointers or
+ * largest histogram of a call without a workspace); bad pointers or
  * shapes with QPE_ERR_ARG. The first call on each device looks up the
  * scratch's device address (cudaGetSymbolAddress); make that first call
  * outside any stream capture. All calls on a device share the scratch: two
