@@ -660,7 +660,7 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
           T.nitems = (int)bm.tc_split.size() - T.item_off;
           if (T.nitems > 0) bm.tc_rounds.push_back(T);
         }
-        for (int dclass : {2, 4, 8, 16, 32, 64}) {
+        for (int dclass : {qpe::kFewRowsClass, 2, 4, 8, 16, 32, 64}) {
           qpe::DblRound R{};
           R.j = j;
           R.dclass = dclass;
@@ -668,7 +668,9 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
           int64_t tiles = 0;
           for (int i : pl) {
             const Instance& in = p->inst[i];
-            if (in.nmeas <= j || on_tc(in, j) || on_oz(in, j) || std::min<int64_t>(in.d, 64) != dclass) continue;
+            if (in.nmeas <= j || on_tc(in, j) || on_oz(in, j)) continue;
+            const bool few = qpe::few_rows(int64_t(1) << j, in.d);
+            if ((few ? qpe::kFewRowsClass : (int)std::min<int64_t>(in.d, 64)) != dclass) continue;
             int BM = 0, BN = 0;
             qpe::doubling_tile((int)in.d, &BM, &BN);
             qpe::DblItem<C> it{};
@@ -677,7 +679,8 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
             it.M = int64_t(1) << j;
             it.d = (int)in.d;
             it.tile0 = tiles;
-            tiles += ((it.M + BM - 1) / BM) * (in.d / BN);
+            tiles += few ? qpe::few_rows_shape((int)it.M, it.d, (int)sizeof(C)).ctas
+                         : ((it.M + BM - 1) / BM) * (in.d / BN);
             push_bytes(bm.dbl_items, &it, sizeof(it));
           }
           R.nitems = (int)(bm.dbl_items.size() / sizeof(qpe::DblItem<C>)) - R.item_off;
@@ -941,7 +944,7 @@ qpe_status enqueue_batched(qpe_plan_t p, int64_t* launches) {
         for (const qpe::DblRound& R : bm.dbl_rounds)
           if (R.j == j &&
               !chk(qpe::launch_doubling_grouped<C>(reinterpret_cast<const qpe::DblItem<C>*>(ws + bm.off_dbl) + R.item_off,
-                                                   R.nitems, R.tiles, R.dclass, p->stream)))
+                                                   R.nitems, R.tiles, R.dclass, R.j, p->stream)))
             return false;
         for (const qpe::GateRound& G : bm.gate_rounds)
           if (G.j == j &&

@@ -195,6 +195,36 @@ __device__ __forceinline__ void merge_partial(Partial& m, const Partial& o) {
   m.wsum += o.wsum;
   m.psum += o.psum;
 }
+// Butterfly reduce-scatter of NV values over the lanes whose index bits below
+// 2 O differ: each step keeps half of the values (the upper half on lanes with
+// bit O set) and adds the partner's copy of that half. With NV >= lanes, lane
+// li ends holding the sums for indices yb0 .. yb0 + NV / lanes - 1; with fewer
+// values than lanes the remaining steps are plain all-reduce steps.
+template <int O, int NV, typename A, int N>
+__device__ __forceinline__ void reduce_scatter_step(A (&v)[N], int li, int& yb0) {
+  if constexpr (O >= 1) {
+    if constexpr (NV > 1) {
+      constexpr int H = NV / 2;
+      const bool up = (li & O) != 0;
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const A send = up ? v[j] : v[j + H];
+        const A keep = up ? v[j + H] : v[j];
+        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+      }
+      if (up) yb0 += H;
+      reduce_scatter_step<O / 2, H>(v, li, yb0);
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+      reduce_scatter_step<O / 2, 1>(v, li, yb0);
+    }
+  }
+}
+template <int O, int NV, typename A, int N>
+__device__ __forceinline__ void reduce_scatter(A (&v)[N], int li, int& yb0) {
+  reduce_scatter_step<O, NV>(v, li, yb0);
+}
+
 // parts[0 .. count) merged by one CTA of 256 threads in a fixed order (the
 // result is deterministic); every thread must call it; thread 0 gets the result.
 __device__ __forceinline__ Partial reduce_partials_256(const Partial* __restrict__ parts, int count) {
@@ -360,6 +390,31 @@ struct InitItem {
   double scale;
   int d, pad;
 };
+// A doubling level of M rows on few_rows_kernel: CTAs of 8 warps, each warp a
+// block of TM x 4 outputs (TM = min(M, 4)); ks warps share a block's inner
+// index, wm x wn blocks per CTA.
+struct FewShape {
+  int ks, wm, wn;
+  int64_t ctas;
+};
+constexpr int kFewRowsTiles = 152;
+constexpr int kFewRowsClass = 0;  // DblRound::dclass of such a level
+__host__ __device__ inline FewShape few_rows_shape(int M, int d, int esize) {
+  const int tm = M < 4 ? M : 4;
+  const int loads = d / (512 / esize);  // 16-byte loads of a warp along the inner index
+  // the inner index is shared until there are 16 warps for each of 152 SMs or a
+  // warp is left with two loads
+  FewShape f{1, 1, 1, 0};
+  const int64_t blocks = (int64_t)((M + tm - 1) / tm) * (d / 4);
+  while (f.ks < 8 && blocks * f.ks < 152 * 16 && loads / (2 * f.ks) >= 2) f.ks *= 2;
+  f.wm = M >= 8 && f.ks <= 4 ? 2 : 1;
+  f.wn = 8 / f.ks / f.wm;
+  f.ctas = (int64_t)((M + tm * f.wm - 1) / (tm * f.wm)) * (d / (4 * f.wn));
+  return f;
+}
+// Levels whose 64 x 64 tiles would leave SMs idle
+inline bool few_rows(int64_t M, int64_t d) { return d >= 64 && ((M + 63) / 64) * (d / 64) < kFewRowsTiles; }
+
 template <typename C>
 struct DblItem {  // rows [M, 2M) = rows [0, M) x P^T
   C* S;
@@ -641,7 +696,7 @@ template <typename C> int level_occupancy(int logd, int r);
 // The batched plain schedule's grouped launches (one per step across instances).
 template <typename C> int launch_init_grouped(const InitItem<C>* items, int nitems, cudaStream_t s);
 template <typename C>
-int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, int dclass, cudaStream_t s);
+int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, int dclass, int j, cudaStream_t s);
 template <typename C>
 int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, cudaStream_t s);
 template <typename C> int launch_reduce_grouped(const RedItem<C>* items, int nitems, int64_t blocks, cudaStream_t s);

@@ -296,6 +296,120 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
                                                           (int)(t % nby));
 }
 
+// Doubling levels of few rows: out_row(M + r)[i] = sum_c P[i][c] S[r][c] for r < M.
+//
+// What bounds it: a 64 x 64 tile with the whole inner dimension gives such a
+// level d / 64 CTAs (16 of 152 SMs at d = 1024), 64 / M of their rows padding, and
+// a chain of d / 8 barriers. Here a warp owns a TM x TN block of outputs (TM rows
+// of S, TN rows of P, each read along the inner index in 16-byte loads by the
+// warp's lanes), KS warps of a CTA share the inner index where the block count
+// alone leaves SMs idle, and the lanes' partial sums meet in one shuffle
+// reduce-scatter: no barrier in the loop, no padding for M >= TM, every SM busy
+// from M d >= 152 x 16 outputs on. The rule that picks it is few_rows().
+constexpr int kFewWarps = 8, kFewTN = 4;
+
+template <int TM>
+__device__ __forceinline__ void few_rows_acc(const float2* const (&a)[TM], const float2* const (&b)[kFewTN], int c,
+                                             float2 (&acc)[TM][kFewTN]) {
+  float4 va[TM], vb[kFewTN];
+#pragma unroll
+  for (int t = 0; t < TM; ++t) va[t] = *reinterpret_cast<const float4*>(a[t] + 2 * c);
+#pragma unroll
+  for (int n = 0; n < kFewTN; ++n) vb[n] = __ldg(reinterpret_cast<const float4*>(b[n] + 2 * c));
+#pragma unroll
+  for (int t = 0; t < TM; ++t)
+#pragma unroll
+    for (int n = 0; n < kFewTN; ++n) {
+      cfma(acc[t][n], make_float2(va[t].x, va[t].y), make_float2(vb[n].x, vb[n].y));
+      cfma(acc[t][n], make_float2(va[t].z, va[t].w), make_float2(vb[n].z, vb[n].w));
+    }
+}
+template <int TM>
+__device__ __forceinline__ void few_rows_acc(const double2* const (&a)[TM], const double2* const (&b)[kFewTN], int c,
+                                             double2 (&acc)[TM][kFewTN]) {
+  double2 va[TM], vb[kFewTN];
+#pragma unroll
+  for (int t = 0; t < TM; ++t) va[t] = a[t][c];
+#pragma unroll
+  for (int n = 0; n < kFewTN; ++n) vb[n] = ld(b[n] + c);
+#pragma unroll
+  for (int t = 0; t < TM; ++t)
+#pragma unroll
+    for (int n = 0; n < kFewTN; ++n) cfma(acc[t][n], va[t], vb[n]);
+}
+
+// CTA `cta` of a level (few_rows_shape(M, d) gives their number)
+template <typename C, int TM>
+__device__ __forceinline__ void few_rows_cta(C* S, const C* __restrict__ P, int M, int d, int64_t cta) {
+  using R_t = typename real_of<C>::type;
+  constexpr int NV = 2 * TM * kFewTN;                    // reals of a warp's block
+  constexpr int LC = 32 * 16 / (int)sizeof(C);           // inner elements of one load by a warp
+  __shared__ R_t red[kFewWarps][NV];
+  const FewShape f = few_rows_shape(M, d, (int)sizeof(C));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ks = warp % f.ks, blk = warp / f.ks;         // inner share, output block of the CTA
+  const int wm = blk % f.wm, wn = blk / f.wm;
+  const int ncols = d / (kFewTN * f.wn);                 // CTAs along the columns
+  const int r0 = ((int)(cta / ncols) * f.wm + wm) * TM;
+  const int i0 = ((int)(cta % ncols) * f.wn + wn) * kFewTN;
+  const C* a[TM];
+  const C* b[kFewTN];
+#pragma unroll
+  for (int t = 0; t < TM; ++t) a[t] = S + (int64_t)(r0 + t < M ? r0 + t : M - 1) * d;  // padding repeats a row
+#pragma unroll
+  for (int n = 0; n < kFewTN; ++n) b[n] = P + (int64_t)(i0 + n) * d;
+  C acc[TM][kFewTN];
+#pragma unroll
+  for (int t = 0; t < TM; ++t)
+#pragma unroll
+    for (int n = 0; n < kFewTN; ++n) acc[t][n] = mk((R_t)0, (R_t)0);
+  const int steps = d / (LC * f.ks);
+#pragma unroll 2
+  for (int k = 0; k < steps; ++k) few_rows_acc<TM>(a, b, (ks * steps + k) * 32 + lane, acc);
+  R_t v[NV];
+#pragma unroll
+  for (int t = 0; t < TM; ++t)
+#pragma unroll
+    for (int n = 0; n < kFewTN; ++n) {
+      v[2 * (t * kFewTN + n)] = acc[t][n].x;
+      v[2 * (t * kFewTN + n) + 1] = acc[t][n].y;
+    }
+  int at = 0;
+  reduce_scatter<16, NV>(v, lane, at);
+  constexpr int PER = NV >= 32 ? NV / 32 : 1;            // sums a lane holds
+  constexpr int DUP = NV >= 32 ? 1 : 32 / NV;            // lanes that hold the same sum
+  if (lane % DUP == 0) {
+#pragma unroll
+    for (int j = 0; j < PER; ++j) red[warp][at + j] = v[j];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < (kFewWarps / f.ks) * NV; e += 32 * kFewWarps) {
+    const int ob = e / NV, q = e % NV;                   // output block of the CTA, real within it
+    R_t s = red[ob * f.ks][q];
+    for (int z = 1; z < f.ks; ++z) s += red[ob * f.ks + z][q];
+    const int row = ((int)(cta / ncols) * f.wm + ob % f.wm) * TM + q / (2 * kFewTN);
+    const int col = ((int)(cta % ncols) * f.wn + ob / f.wm) * kFewTN;
+    if (row < M) reinterpret_cast<R_t*>(S + (int64_t)(M + row) * d + col)[q % (2 * kFewTN)] = s;
+  }
+}
+
+template <typename C, int TM>
+__global__ void __launch_bounds__(32 * kFewWarps) few_rows_kernel(C* S, const C* __restrict__ P, int M, int d) {
+  pdl_begin();
+  few_rows_cta<C, TM>(S, P, M, d, blockIdx.x);
+  pdl_trigger();
+}
+
+// one such level for every listed instance (all of the same M)
+template <typename C, int TM>
+__global__ void __launch_bounds__(32 * kFewWarps)
+    few_rows_grouped_kernel(const DblItem<C>* __restrict__ items, int nitems) {
+  pdl_begin();
+  const DblItem<C> it = items[find_item(items, nitems, blockIdx.x)];
+  few_rows_cta<C, TM>(it.S, it.P, (int)it.M, it.d, blockIdx.x - it.tile0);
+  pdl_trigger();
+}
+
 // ------------------------------------------------------------------ fft
 // One decimation-in-frequency pass over the middle axis of X viewed as
 // [B][R][Q] (Q = L * d contiguous elements): for each block and each of the Q
@@ -936,6 +1050,21 @@ static int launch_rows_times_pt(C* S, const C* P, int64_t M, int d, Rows rows, c
   return err == cudaSuccess ? 1 : -1;
 }
 
+// One doubling level on the CUDA cores.
+template <typename C>
+static int launch_doubling(C* S, const C* P, int64_t M, int d, cudaStream_t s) {
+  if (!few_rows(M, d)) return launch_rows_times_pt<C>(S, P, M, d, DoublingRows{M}, s);
+  const dim3 grid((unsigned)few_rows_shape((int)M, d, (int)sizeof(C)).ctas), block(32 * kFewWarps);
+  cudaError_t e;
+  if (M == 1)
+    e = launch_k(few_rows_kernel<C, 1>, grid, block, 0, s, S, P, (int)M, d);
+  else if (M == 2)
+    e = launch_k(few_rows_kernel<C, 2>, grid, block, 0, s, S, P, (int)M, d);
+  else
+    e = launch_k(few_rows_kernel<C, 4>, grid, block, 0, s, S, P, (int)M, d);
+  return e == cudaSuccess ? 1 : -1;
+}
+
 template <typename C>
 int launch_sweep(const Instance& in, char* ws, bool gate_mode, cudaStream_t s, int prec) {
   const bool tc = prec == QPE_C64_TF32X3 || prec == QPE_C64_FP16X2;
@@ -956,7 +1085,7 @@ int launch_sweep(const Instance& in, char* ws, bool gate_mode, cudaStream_t s, i
     // n - sh qubits over the local rows (local row i = U^(r + G i) psi)
     const int sh = in.shard_log;
     for (int j = 0; j < sh; ++j) {
-      const int r = launch_rows_times_pt<C>(S, P + j * dd, int64_t(1) << j, (int)in.d, DoublingRows{int64_t(1) << j}, s);
+      const int r = launch_doubling<C>(S, P + j * dd, int64_t(1) << j, (int)in.d, s);
       if (r < 0) return -1;
       launches += r;
     }
@@ -971,8 +1100,7 @@ int launch_sweep(const Instance& in, char* ws, bool gate_mode, cudaStream_t s, i
       else if (sizeof(C) == 16 && in.oz_gates && (int64_t(1) << j) >= 128)
         r = launch_oz_gate_level(in, ws, j, sh, s);
       else
-        r = launch_rows_times_pt<C>(S, P + (j + sh) * dd, int64_t(1) << j, (int)in.d, DoublingRows{int64_t(1) << j},
-                                    s);
+        r = launch_doubling<C>(S, P + (j + sh) * dd, int64_t(1) << j, (int)in.d, s);
       if (r < 0) return -1;
       launches += r;
     }
@@ -994,7 +1122,7 @@ int launch_sweep(const Instance& in, char* ws, bool gate_mode, cudaStream_t s, i
     else if (sizeof(C) == 16 && in.oz_gates && (int64_t(1) << j) >= 128)
       r = launch_oz_gate_level(in, ws, j, 0, s);  // FP64: exact digit products on the tensor cores
     else
-      r = launch_rows_times_pt<C>(S, P + j * dd, int64_t(1) << j, (int)in.d, DoublingRows{int64_t(1) << j}, s);
+      r = launch_doubling<C>(S, P + j * dd, int64_t(1) << j, (int)in.d, s);
     if (r < 0) return -1;
     launches += r;
   }
@@ -1098,12 +1226,22 @@ int launch_init_grouped(const InitItem<C>* items, int nitems, cudaStream_t s) {
   return launch_k(init_grouped_kernel<C>, dim3((unsigned)nitems), dim3(256), 0, s, items) == cudaSuccess ? 1 : -1;
 }
 
-// one doubling round for the items of one tile class (d, or 64 for d >= 64)
+// one doubling round for the items of one tile class (d, 64 for d >= 64, or
+// kFewRowsClass for the levels few_rows() takes)
 template <typename C>
-int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, int dclass, cudaStream_t s) {
+int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, int dclass, int j, cudaStream_t s) {
   if (nitems <= 0) return 0;
   cudaError_t e;
+  const dim3 few(32 * kFewWarps);
   switch (dclass) {
+    case kFewRowsClass:
+      if (j == 0)
+        e = launch_k(few_rows_grouped_kernel<C, 1>, dim3((unsigned)tiles), few, 0, s, items, nitems);
+      else if (j == 1)
+        e = launch_k(few_rows_grouped_kernel<C, 2>, dim3((unsigned)tiles), few, 0, s, items, nitems);
+      else
+        e = launch_k(few_rows_grouped_kernel<C, 4>, dim3((unsigned)tiles), few, 0, s, items, nitems);
+      break;
     case 2: e = launch_k(doubling_grouped_kernel<C, 256, 2, 2, 2, 1>, dim3((unsigned)tiles), dim3(256), 0, s, items, nitems); break;
     case 4: e = launch_k(doubling_grouped_kernel<C, 256, 4, 4, 4, 1>, dim3((unsigned)tiles), dim3(256), 0, s, items, nitems); break;
     case 8: e = launch_k(doubling_grouped_kernel<C, 256, 8, 8, 4, 2>, dim3((unsigned)tiles), dim3(256), 0, s, items, nitems); break;
@@ -1213,7 +1351,7 @@ template int launch_fft<double2>(const Instance&, char*, cudaStream_t);
 template int launch_reduce<float2>(const Instance&, char*, cudaStream_t);
 #define QPE_GROUPED_INST(C)                                                                             \
   template int launch_init_grouped<C>(const InitItem<C>*, int, cudaStream_t);                          \
-  template int launch_doubling_grouped<C>(const DblItem<C>*, int, int64_t, int, cudaStream_t);         \
+  template int launch_doubling_grouped<C>(const DblItem<C>*, int, int64_t, int, int, cudaStream_t);    \
   template int launch_fft_grouped<C>(const FftItem<C>*, int, int64_t, size_t, cudaStream_t);           \
   template int launch_reduce_grouped<C>(const RedItem<C>*, int, int64_t, cudaStream_t);
 QPE_GROUPED_INST(float2)

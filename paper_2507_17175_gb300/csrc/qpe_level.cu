@@ -229,36 +229,6 @@ __device__ __forceinline__ void dft_r(C (&x)[N], int r) {
   }
 }
 
-// Butterfly reduce-scatter of NV values over the lanes whose index bits below
-// 2 O differ: each step keeps half of the values (the upper half on lanes with
-// bit O set) and adds the partner's copy of that half. With NV >= lanes, lane
-// li ends holding the sums for indices yb0 .. yb0 + NV / lanes - 1; with fewer
-// values than lanes the remaining steps are plain all-reduce steps.
-template <int O, int NV, typename A, int N>
-__device__ __forceinline__ void reduce_scatter_step(A (&v)[N], int li, int& yb0) {
-  if constexpr (O >= 1) {
-    if constexpr (NV > 1) {
-      constexpr int H = NV / 2;
-      const bool up = (li & O) != 0;
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const A send = up ? v[j] : v[j + H];
-        const A keep = up ? v[j + H] : v[j];
-        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-      }
-      if (up) yb0 += H;
-      reduce_scatter_step<O / 2, H>(v, li, yb0);
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-      reduce_scatter_step<O / 2, 1>(v, li, yb0);
-    }
-  }
-}
-template <int O, int NV, typename A, int N>
-__device__ __forceinline__ void reduce_scatter(A (&v)[N], int li, int& yb0) {
-  reduce_scatter_step<O, NV>(v, li, yb0);
-}
-
 // ------------------------------------------------------------------ kernel
 // One CTA's share of a level: column group cg, pencil-group iterations
 // it_begin, it_begin + it_step, ... < it_end. MODE != 0 writes this share's
