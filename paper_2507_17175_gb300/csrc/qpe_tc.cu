@@ -76,6 +76,7 @@ using namespace tcg;
 constexpr int kGroupM = 8;
 constexpr int kKPC = 8;  // K-blocks per cross-term chunk
 constexpr int kMS = 2;   // hi.hi drains per K-block (every 2 MMA instructions)
+static_assert(kMS % 2 == 0, "the main buffers alternate within a K-block");
 constexpr int kTcDrainWarps = 8;  // 4 lane quarters x 2 column halves
 
 template <int KIND, int BN>
@@ -161,64 +162,59 @@ __device__ __forceinline__ void tc_gemm_tile(const CUtensorMap* mapAhi, const CU
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc<KIND, BN>();
-      for (int kb = 0; kb < kblocks; ++kb) {
-        const int cx = kb / kKPC, bx = cx & 1;    // cross chunk and its buffer
-        const bool cx_first = (kb % kKPC) == 0;
-        const bool cx_last = (kb % kKPC) == kKPC - 1 || kb == kblocks - 1;
-        if (cx_first && cx >= 2 && !mbar_wait(&cross_empty[bx], ((cx >> 1) - 1) & 1)) {
-          atomicExch(&fail, 1);
-          break;
-        }
-        const int st = kb % QS;
-        if (!mbar_wait(&full_bar[st], (kb / QS) & 1)) {
-          atomicExch(&fail, 1);
-          break;
-        }
+    // the whole warp runs the loop; one elected lane issues
+    const uint32_t idesc = make_idesc<KIND, BN>();
+    const uint64_t ring_desc = sw128_desc(smem_u32(ring));
+    int st = 0;
+    uint32_t phase = 0;
+    for (int kb = 0; kb < kblocks; ++kb) {
+      const int cx = kb / kKPC, bx = cx & 1;    // cross chunk and its buffer
+      const bool cx_first = (kb % kKPC) == 0;
+      const bool cx_last = (kb % kKPC) == kKPC - 1 || kb == kblocks - 1;
+      bool ok = !(cx_first && cx >= 2) || mbar_wait_warp(&cross_empty[bx], ((cx >> 1) - 1) & 1);
+      ok = ok && mbar_wait_warp(&full_bar[st], phase);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint64_t ah = ring_desc + (uint64_t)(st * (STAGE_BYTES >> 4));
+      const uint64_t al = ah + (A_BYTES >> 4), bh = ah + (2 * A_BYTES >> 4), bl = bh + (B_BYTES >> 4);
+      // hi.hi: kMS groups of 4 / kMS instructions, each group into its own main buffer
+#pragma unroll
+      for (int gs = 0; gs < kMS; ++gs) {
+        const int j = kb * kMS + gs;
+        constexpr int per = 4 / kMS;
+        const int bm = gs & 1;  // kMS is even: j & 1
+        ok = ok && (j < 2 || mbar_wait_warp(&main_empty[bm], ((j >> 1) - 1) & 1));
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = smem_u32(ring + st * STAGE_BYTES);
-        bool ok = true;
-        {  // hi.hi: kMS groups of 4 / kMS instructions, each group into its own main buffer
-          const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + 2 * A_BYTES);
-          for (int gs = 0; gs < kMS; ++gs) {
-            const int j = kb * kMS + gs, bm = j & 1;
-            if (j >= 2 && !mbar_wait(&main_empty[bm], ((j >> 1) - 1) & 1)) {
-              ok = false;
-              break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4 / kMS; ++kk) {
-              const int k = gs * (4 / kMS) + kk;
-              umma_k<KIND>(tmem + (uint32_t)(bm * BN), ad + 2 * k, bd + 2 * k, idesc, kk == 0 ? 0u : 1u);
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&main_full[bm]))
-                         : "memory");
-          }
+          for (int kk = 0; kk < per; ++kk)
+            umma_k<KIND>(tmem + (uint32_t)(bm * BN), ah + 2 * (gs * per + kk), bh + 2 * (gs * per + kk), idesc,
+                         kk == 0 ? 0u : 1u);
+          umma_commit(&main_full[bm]);
         }
-        if (!ok) {
-          atomicExch(&fail, 1);
-          break;
-        }
-        for (int pr = 1; pr < 3; ++pr) {  // (hi, lo), (lo, hi) into the cross buffer
-          const uint64_t ad = sw128_desc(pr == 2 ? sa + A_BYTES : sa);
-          const uint64_t bd = sw128_desc(sa + 2 * A_BYTES + (pr == 1 ? B_BYTES : 0));
-          const uint32_t acc_addr = tmem + (uint32_t)((2 + bx) * BN);
+      }
+      if (!ok) {
+        atomicExch(&fail, 1);
+        break;
+      }
+      // (hi, lo), (lo, hi) into the cross buffer, 32 bytes of K per instruction
+      const uint32_t acc_addr = tmem + (uint32_t)((2 + bx) * BN);
+      if (cx_first) {
+        if (elect_one()) umma_k<KIND>(acc_addr, ah, bl, idesc, 0u);
+      } else {
+        if (elect_one()) umma_k<KIND>(acc_addr, ah, bl, idesc, 1u);
+      }
+      if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {  // 32 bytes of K per instruction
-            const bool fresh = k == 0 && pr == 1 && cx_first;
-            umma_k<KIND>(acc_addr, ad + 2 * k, bd + 2 * k, idesc, fresh ? 0u : 1u);
-          }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(&empty_bar[st]))
-                     : "memory");
-        if (cx_last)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(&cross_full[bx]))
-                       : "memory");
+        for (int k = 1; k < 4; ++k) umma_k<KIND>(acc_addr, ah + 2 * k, bl + 2 * k, idesc, 1u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) umma_k<KIND>(acc_addr, al + 2 * k, bh + 2 * k, idesc, 1u);
+        umma_commit(&empty_bar[st]);
+        if (cx_last) umma_commit(&cross_full[bx]);
+      }
+      if (++st == QS) {
+        st = 0;
+        phase ^= 1u;
       }
     }
   } else {
@@ -698,45 +694,64 @@ __device__ __forceinline__ bool oz_window_end(int kb, int kblocks) {
   return ((kb + 1 + oz_off<W>()) & (oz_win<W>() - 1)) == 0 || kb + 1 == kblocks;
 }
 
-// The MMAs of A digit S against B digits T .. 6 - S (one K-block): pair
-// (S, T) into the accumulator of weight S + T, four K = 16 steps. The first
-// pair of a window (S = 0) overwrites the accumulator, after waiting for the
-// drain of the window before. False if that wait runs out.
+// Pair (S, T): four K = 16 steps into the accumulator of weight S + T; FRESH
+// overwrites it.
+template <int S, int T, bool FRESH>
+__device__ __forceinline__ void oz_mma_pair(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc) {
+  const uint64_t bd = bd0 + (uint64_t)(T * (kOzB >> 4));
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    umma_k<kTcBF16>(tmem + (uint32_t)((S + T) * kOzBN), ad + 2 * k, bd + 2 * k, idesc, (FRESH && k == 0) ? 0u : 1u);
+}
 template <int S, int T>
-__device__ __forceinline__ bool oz_mma_pairs(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc, int kb,
-                                             uint64_t* acc_empty) {
+__device__ __forceinline__ void oz_mma_pairs(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc) {
   if constexpr (S + T < kOzS) {
-    constexpr int w = S + T;
-    bool fresh = false;
-    if constexpr (S == 0) {
-      fresh = oz_window_start<w>(kb);
-      if (fresh && kb > 0) {
-        if (!mbar_wait(&acc_empty[w], (oz_window<w>(kb) - 1) & 1)) return false;
+    oz_mma_pair<S, T, false>(tmem, ad, bd0, idesc);
+    oz_mma_pairs<S, T + 1>(tmem, ad, bd0, idesc);
+  }
+}
+
+// Digit 0's pairs: pair (0, T) is the first of weight T in a K-block. At the
+// start of a window it waits for the drain of the window before and overwrites
+// the accumulator. False if that wait runs out.
+template <int T>
+__device__ __forceinline__ bool oz_mma_first(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc, int kb,
+                                             uint64_t* acc_empty) {
+  if constexpr (T < kOzS) {
+    if (oz_window_start<T>(kb)) {
+      if (kb > 0) {
+        if (!mbar_wait_warp(&acc_empty[T], (oz_window<T>(kb) - 1) & 1)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
+      if (elect_one()) oz_mma_pair<0, T, true>(tmem, ad, bd0, idesc);
+    } else if (elect_one()) {
+      oz_mma_pair<0, T, false>(tmem, ad, bd0, idesc);
     }
-    const uint64_t bd = bd0 + (uint64_t)(T * (kOzB >> 4));
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      umma_k<kTcBF16>(tmem + (uint32_t)(w * kOzBN), ad + 2 * k, bd + 2 * k, idesc, (fresh && k == 0) ? 0u : 1u);
-    return oz_mma_pairs<S, T + 1>(tmem, ad, bd0, idesc, kb, acc_empty);
+    return oz_mma_first<T + 1>(tmem, ad, bd0, idesc, kb, acc_empty);
   }
   return true;
 }
 
-// A digits S .. 6 of one K-block: wait for the digit's ring stage, its pairs,
-// release the stage, and signal weight S complete at the end of its window.
+// A digits S .. 6 of one K-block (the whole warp; one elected lane issues):
+// wait for the digit's ring stage, its pairs, release the stage, and signal
+// weight S complete at the end of its window.
 template <int S>
 __device__ __forceinline__ bool oz_mma_digits(uint32_t tmem, uint64_t a_desc0, uint64_t bd0, uint32_t idesc, int kb,
                                               int kblocks, int& stage, uint32_t& phase, uint64_t* a_full,
                                               uint64_t* a_empty, uint64_t* acc_full, uint64_t* acc_empty) {
   if constexpr (S < kOzS) {
-    if (!mbar_wait(&a_full[stage], phase)) return false;
+    if (!mbar_wait_warp(&a_full[stage], phase)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint64_t ad = a_desc0 + (uint64_t)(stage * (kOzA >> 4));
-    if (!oz_mma_pairs<S, 0>(tmem, ad, bd0, idesc, kb, acc_empty)) return false;
-    umma_commit(&a_empty[stage]);
-    if (oz_window_end<S>(kb, kblocks)) umma_commit(&acc_full[S]);  // weight S is complete
+    if constexpr (S == 0) {
+      if (!oz_mma_first<0>(tmem, ad, bd0, idesc, kb, acc_empty)) return false;
+    }
+    const bool done = oz_window_end<S>(kb, kblocks);  // weight S is complete
+    if (elect_one()) {
+      if constexpr (S > 0) oz_mma_pairs<S, 0>(tmem, ad, bd0, idesc);
+      umma_commit(&a_empty[stage]);
+      if (done) umma_commit(&acc_full[S]);
+    }
     if (++stage == kOzAStages) {
       stage = 0;
       phase ^= 1u;
@@ -880,30 +895,28 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc<kTcBF16, kOzBN>();
-      const uint64_t a_desc0 = sw128_desc(smem_u32(aring)), b_desc0 = sw128_desc(smem_u32(bset));
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int kb = 0; kb < kblocks; ++kb) {
-        const int bb = kb & 1;
-        if (!mbar_wait(&b_full[bb], (kb >> 1) & 1)) {
-          atomicExch(&fail, 1);
-          break;
-        }
+    const uint32_t idesc = make_idesc<kTcBF16, kOzBN>();
+    const uint64_t a_desc0 = sw128_desc(smem_u32(aring)), b_desc0 = sw128_desc(smem_u32(bset));
+    int stage = 0;
+    uint32_t phase = 0;
+    for (int kb = 0; kb < kblocks; ++kb) {
+      const int bb = kb & 1;
+      bool ok = mbar_wait_warp(&b_full[bb], (kb >> 1) & 1);
+      if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t bd0 = b_desc0 + (uint64_t)(bb * (kOzBSet >> 4));
-        if (!oz_mma_digits<0>(tmem, a_desc0, bd0, idesc, kb, kblocks, stage, phase, a_full, a_empty, acc_full,
-                              acc_empty)) {
-          atomicExch(&fail, 1);
-          break;
-        }
-        umma_commit(&b_empty[bb]);
+        ok = oz_mma_digits<0>(tmem, a_desc0, bd0, idesc, kb, kblocks, stage, phase, a_full, a_empty, acc_full,
+                              acc_empty);
       }
-      // every MMA issued has finished before tensor memory is released
-      umma_commit(&mma_done);
-      if (!mbar_wait(&mma_done, 0)) atomicExch(&fail, 1);
+      if (!ok) {
+        atomicExch(&fail, 1);
+        break;
+      }
+      if (elect_one()) umma_commit(&b_empty[bb]);
     }
+    // every MMA issued has finished before tensor memory is released
+    if (elect_one()) umma_commit(&mma_done);
+    if (!mbar_wait_warp(&mma_done, 0)) atomicExch(&fail, 1);
   } else {
     const int q = warp & 3;          // tensor-memory lane quarter
     const int h = (warp - 2) >> 2;   // column half

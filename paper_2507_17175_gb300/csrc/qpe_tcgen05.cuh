@@ -60,6 +60,28 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
+// One lane of a converged warp (the same one each time). The tcgen05.mma
+// operands live in uniform registers: code under `if (threadIdx... == 0)` makes the
+// compiler move every descriptor there through the vector registers, 50 to 100
+// clocks an MMA; a loop that all 32 lanes run, with only the MMAs of a group
+// under elect_one(), keeps them uniform (measured: 32 clocks for M = 128, N = 64
+// with A in tensor memory, the tensor pipe's own rate; 48 with A in shared memory,
+// its read rate).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(p));
+  return p != 0;
+}
+
+// mbar_wait by a converged warp: every lane polls, one answer for all
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity)) != 0;
+}
+
 // Shared-memory matrix descriptor for a K-major, 128-byte-swizzled tile:
 // start address >> 4, leading offset 16 B (unused for swizzled K-major),
 // stride offset 1024 B between 8-row groups, descriptor version 1,
