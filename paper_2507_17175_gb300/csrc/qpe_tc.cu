@@ -174,7 +174,7 @@ __device__ __forceinline__ void tc_gemm_tile(const CUtensorMap* mapAhi, const CU
       bool ok = !(cx_first && cx >= 2) || mbar_wait_warp(&cross_empty[bx], ((cx >> 1) - 1) & 1);
       ok = ok && mbar_wait_warp(&full_bar[st], phase);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ah = ring_desc + (uint64_t)(st * (STAGE_BYTES >> 4));
+      const uint64_t ah = ring_desc + (uint64_t)(__shfl_sync(0xffffffffu, st, 0) * (STAGE_BYTES >> 4));
       const uint64_t al = ah + (A_BYTES >> 4), bh = ah + (2 * A_BYTES >> 4), bl = bh + (B_BYTES >> 4);
       // hi.hi: kMS groups of 4 / kMS instructions, each group into its own main buffer
 #pragma unroll
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows_grouped_kernel(const RowSli
 // One CTA per 128 x 64 tile of out (rows m0.. of E, columns n0.. < d).
 // K-block by K-block (64 elements of K), every digit tile is loaded once: the
 // seven B digit tiles of the K-block (resident, two buffers) and the seven A
-// digit tiles one after another through a ring; A digit s meets B digits
+// digit tiles, each refilled once its pairs are done; A digit s meets B digits
 // t = 0 .. 6 - s, and pair (s, t) goes into the tensor-memory accumulator of
 // weight w = s + t (64 columns each, 448 in all). Weight w is complete for the
 // K-block once A digit w has been used, so the weights finish in order and
@@ -664,7 +664,6 @@ __global__ void __launch_bounds__(256) oz_slice_rows_grouped_kernel(const RowSli
 // val = hi 2^-32 + lo 2^-64 and out = val 2^(tau_m + sigma_n + 2).
 // Warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the MMAs.
 constexpr int kOzBN = 64;
-constexpr int kOzAStages = 6;
 constexpr int kOzThreads = 320;
 constexpr int kOzA = kBM * 128;              // one A digit tile, 16 KiB
 constexpr int kOzB = kOzBN * 128;            // one B digit tile, 8 KiB
@@ -733,32 +732,44 @@ __device__ __forceinline__ bool oz_mma_first(uint32_t tmem, uint64_t ad, uint64_
 }
 
 // A digits S .. 6 of one K-block (the whole warp; one elected lane issues):
-// wait for the digit's ring stage, its pairs, release the stage, and signal
-// weight S complete at the end of its window.
+// wait for the digit's tile, its pairs, release the tile, and signal weight S
+// complete at the end of its window. Every descriptor is a constant away from
+// a loop invariant: with a ring stage computed at run time an MMA took 72
+// clocks to issue against the 48 its operands take to read.
 template <int S>
 __device__ __forceinline__ bool oz_mma_digits(uint32_t tmem, uint64_t a_desc0, uint64_t bd0, uint32_t idesc, int kb,
-                                              int kblocks, int& stage, uint32_t& phase, uint64_t* a_full,
-                                              uint64_t* a_empty, uint64_t* acc_full, uint64_t* acc_empty) {
+                                              int kblocks, uint64_t* a_full, uint64_t* a_empty, uint64_t* acc_full,
+                                              uint64_t* acc_empty) {
   if constexpr (S < kOzS) {
-    if (!mbar_wait_warp(&a_full[stage], phase)) return false;
+    if (!mbar_wait_warp(&a_full[S], kb & 1)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint64_t ad = a_desc0 + (uint64_t)(stage * (kOzA >> 4));
+    const uint64_t ad = a_desc0 + (uint64_t)(S * (kOzA >> 4));
     if constexpr (S == 0) {
       if (!oz_mma_first<0>(tmem, ad, bd0, idesc, kb, acc_empty)) return false;
     }
     const bool done = oz_window_end<S>(kb, kblocks);  // weight S is complete
     if (elect_one()) {
       if constexpr (S > 0) oz_mma_pairs<S, 0>(tmem, ad, bd0, idesc);
-      umma_commit(&a_empty[stage]);
+      umma_commit(&a_empty[S]);
       if (done) umma_commit(&acc_full[S]);
     }
-    if (++stage == kOzAStages) {
-      stage = 0;
-      phase ^= 1u;
-    }
-    return oz_mma_digits<S + 1>(tmem, a_desc0, bd0, idesc, kb, kblocks, stage, phase, a_full, a_empty, acc_full,
-                                acc_empty);
+    return oz_mma_digits<S + 1>(tmem, a_desc0, bd0, idesc, kb, kblocks, a_full, a_empty, acc_full, acc_empty);
   }
+  return true;
+}
+
+// One K-block on B buffer BB (the whole warp)
+template <int BB>
+__device__ __forceinline__ bool oz_mma_kblock(uint32_t tmem, uint64_t a_desc0, uint64_t b_desc0, uint32_t idesc,
+                                              int kb, int kblocks, uint64_t* a_full, uint64_t* a_empty,
+                                              uint64_t* b_full, uint64_t* b_empty, uint64_t* acc_full,
+                                              uint64_t* acc_empty) {
+  if (!mbar_wait_warp(&b_full[BB], (kb >> 1) & 1)) return false;
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!oz_mma_digits<0>(tmem, a_desc0, b_desc0 + (uint64_t)(BB * (kOzBSet >> 4)), idesc, kb, kblocks, a_full, a_empty,
+                        acc_full, acc_empty))
+    return false;
+  if (elect_one()) umma_commit(&b_empty[BB]);
   return true;
 }
 
@@ -807,9 +818,9 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
   extern __shared__ __align__(1024) unsigned char smem_dyn[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
-  unsigned char* bset = base;                 // 2 x kOzBSet
-  unsigned char* aring = base + 2 * kOzBSet;  // kOzAStages x kOzA
-  __shared__ uint64_t a_full[kOzAStages], a_empty[kOzAStages], b_full[2], b_empty[2];
+  unsigned char* bset = base;                // 2 x kOzBSet
+  unsigned char* aset = base + 2 * kOzBSet;  // kOzS x kOzA
+  __shared__ uint64_t a_full[kOzS], a_empty[kOzS], b_full[2], b_empty[2];
   __shared__ uint64_t acc_full[kOzS], acc_empty[kOzS], mma_done;
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
@@ -833,7 +844,7 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
   const int kblocks = d2 / 64;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kOzAStages; ++s) {
+    for (int s = 0; s < kOzS; ++s) {
       mbar_init(&a_full[s], 1);
       mbar_init(&a_empty[s], 1);
     }
@@ -863,7 +874,6 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
   int a_issued = 0, b_issued = 0;  // producer: loads issued (to wait for them after a failure)
   if (warp == 0) {
     if (lane == 0) {
-      int it = 0;
       for (int kb = 0; kb < kblocks; ++kb) {
         const int bb = kb & 1;
         if (kb >= 2 && !mbar_wait(&b_empty[bb], ((kb >> 1) - 1) & 1)) {
@@ -876,9 +886,8 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
           tma_load_2d(bset + bb * kOzBSet + t * kOzB, mapB, &b_full[bb], kb * 64, t * ncols + n0);
         ++b_issued;
         bool go = true;
-        for (int s = 0; s < kOzS; ++s, ++it) {
-          const int st = it % kOzAStages;
-          if (it >= kOzAStages && !mbar_wait(&a_empty[st], ((it / kOzAStages) - 1) & 1)) {
+        for (int s = 0; s < kOzS; ++s) {
+          if (kb >= 1 && !mbar_wait(&a_empty[s], (kb - 1) & 1)) {
             atomicExch(&fail, 1);
             go = false;
             break;
@@ -887,8 +896,8 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
             go = false;
             break;
           }
-          mbar_expect_tx(&a_full[st], kOzA);
-          tma_load_2d(aring + st * kOzA, mapA, &a_full[st], kb * 64, s * mrows + m0);
+          mbar_expect_tx(&a_full[s], kOzA);
+          tma_load_2d(aset + s * kOzA, mapA, &a_full[s], kb * 64, s * mrows + m0);
           ++a_issued;
         }
         if (!go) break;
@@ -896,23 +905,15 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
     }
   } else if (warp == 1) {
     const uint32_t idesc = make_idesc<kTcBF16, kOzBN>();
-    const uint64_t a_desc0 = sw128_desc(smem_u32(aring)), b_desc0 = sw128_desc(smem_u32(bset));
-    int stage = 0;
-    uint32_t phase = 0;
-    for (int kb = 0; kb < kblocks; ++kb) {
-      const int bb = kb & 1;
-      bool ok = mbar_wait_warp(&b_full[bb], (kb >> 1) & 1);
-      if (ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t bd0 = b_desc0 + (uint64_t)(bb * (kOzBSet >> 4));
-        ok = oz_mma_digits<0>(tmem, a_desc0, bd0, idesc, kb, kblocks, stage, phase, a_full, a_empty, acc_full,
-                              acc_empty);
-      }
-      if (!ok) {
+    const uint64_t a_desc0 = sw128_desc(smem_u32(aset)), b_desc0 = sw128_desc(smem_u32(bset));
+    for (int kb = 0; kb < kblocks; kb += 2) {
+      if (!oz_mma_kblock<0>(tmem, a_desc0, b_desc0, idesc, kb, kblocks, a_full, a_empty, b_full, b_empty, acc_full,
+                            acc_empty) ||
+          (kb + 1 < kblocks && !oz_mma_kblock<1>(tmem, a_desc0, b_desc0, idesc, kb + 1, kblocks, a_full, a_empty,
+                                                 b_full, b_empty, acc_full, acc_empty))) {
         atomicExch(&fail, 1);
         break;
       }
-      if (elect_one()) umma_commit(&b_empty[bb]);
     }
     // every MMA issued has finished before tensor memory is released
     if (elect_one()) umma_commit(&mma_done);
@@ -962,8 +963,8 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
   __syncthreads();
   if (warp == 0 && lane == 0 && fail) {
     // copies still in flight land before the CTA's shared memory is released
-    const int na = a_issued < kOzAStages ? a_issued : kOzAStages;
-    for (int j = a_issued - na; j < a_issued; ++j) mbar_wait(&a_full[j % kOzAStages], (j / kOzAStages) & 1);
+    const int na = a_issued < kOzS ? a_issued : kOzS;
+    for (int j = a_issued - na; j < a_issued; ++j) mbar_wait(&a_full[j % kOzS], (j / kOzS) & 1);
     const int nb = b_issued < 2 ? b_issued : 2;
     for (int j = b_issued - nb; j < b_issued; ++j) mbar_wait(&b_full[j & 1], (j >> 1) & 1);
   }
@@ -1074,7 +1075,7 @@ size_t tc_smem() {
 }
 
 // two sets of B digit tiles, the A ring, 1 KiB for the alignment
-size_t oz_smem() { return (size_t)2 * kOzBSet + (size_t)kOzAStages * kOzA + 1024; }
+size_t oz_smem() { return (size_t)2 * kOzBSet + (size_t)kOzS * kOzA + 1024; }
 
 }  // namespace
 
