@@ -450,61 +450,64 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
     // buffers in turn; the table's chunk image streams through a ring of
     // kOtBStages stages by bulk copies, kOtBStages - 2 chunks ahead (a stage
     // is refilled once the MMAs of the chunk two back, its last reader, are done).
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc<kTcBF16, 32>();
-      const int64_t first = a.tile_begin + blockIdx.x;
-      const int64_t ntile = first < a.tile_end ? (a.tile_end - first + gridDim.x - 1) / gridDim.x : 0;
-      const int64_t total = ntile * kOtChunks;
-      int64_t issued = 0, g = 0;
-      bool ok = true;
-      auto issue = [&](int64_t gq) {
-        const int st = (int)(gq % kOtBStages);
-        if (gq >= kOtBStages && !mbar_wait(&b_empty[st], (uint32_t)(((gq / kOtBStages) - 1) & 1))) return false;
+    // The whole warp runs the loop and one elected lane issues; the chunks of a
+    // tile and the two digit buffers are unrolled, so that every descriptor is a
+    // constant away from a loop invariant (an MMA issues in 42 clocks, the read
+    // rate of its operands, instead of about 100).
+    const uint32_t idesc = make_idesc<kTcBF16, 32>();
+    const uint64_t a_desc0 = sw128_desc(smem_u32(As)), b_desc0 = sw128_desc(smem_u32(Bs));
+    const int64_t first = a.tile_begin + blockIdx.x;
+    const int64_t ntile = first < a.tile_end ? (a.tile_end - first + gridDim.x - 1) / gridDim.x : 0;
+    const int64_t total = ntile * kOtChunks;
+    int64_t issued = 0, g = 0;
+    bool ok = true;
+    auto issue = [&](int64_t gq) {
+      const int st = (int)(gq % kOtBStages);
+      if (gq >= kOtBStages && !mbar_wait_warp(&b_empty[st], (uint32_t)(((gq / kOtBStages) - 1) & 1))) return false;
+      if (lane == 0) {
         mbar_expect_tx(&b_full[st], kOtBChunk);
         bulk_load(Bs + st * kOtBChunk, a.btab + (size_t)(gq % kOtChunks) * kOtBChunk, kOtBChunk, &b_full[st]);
-        return true;
-      };
-      while (ok && issued < total && issued < kOtBStages - 2) {
-        ok = issue(issued);
-        issued += ok ? 1 : 0;
       }
-      int it = 0;
-      for (int64_t t = first; t < a.tile_end && ok; t += gridDim.x, ++it) {
-        const int ab = it & 1;
-        if (!mbar_wait(&a_full[ab], (it >> 1) & 1) || *vfail) {
-          ok = false;
-          break;
+      return true;
+    };
+    while (ok && issued < total && issued < kOtBStages - 2) {
+      ok = issue(issued);
+      issued += ok ? 1 : 0;
+    }
+    static_assert(kOtChunks % kOtBStages == 0 && kOtChunks % 2 == 0, "a tile's chunks meet fixed stages and buffers");
+    auto tile = [&](uint64_t a0, int ab, int64_t it) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&a_full[ab], (it >> 1) & 1) && !*vfail)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int c = 0; c < kOtChunks; ++c, ++g) {
+        if (issued < total) {
+          if (!issue(issued)) return false;
+          ++issued;
         }
+        constexpr int per = kOtChunks / kOtBStages;  // fills of a stage per tile
+        const int st = c % kOtBStages, buf = c & 1;
+        if (!mbar_wait_warp(&b_full[st], (uint32_t)((it * per + c / kOtBStages) & 1))) return false;
+        if ((it > 0 || c >= 2) && !mbar_wait_warp(&t_empty[buf], (uint32_t)((it * (kOtChunks / 2) + (c >> 1) - 1) & 1)))
+          return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t a0 = sw128_desc(smem_u32(As + ab * kOtABytes));
-        for (int c = 0; c < kOtChunks; ++c, ++g) {
-          if (issued < total) {
-            if (!(ok = issue(issued))) break;
-            ++issued;
-          }
-          const int st = (int)(g % kOtBStages);
-          const int buf = c & 1;
-          if (!mbar_wait(&b_full[st], (uint32_t)((g / kOtBStages) & 1)) ||
-              (g >= 2 && !mbar_wait(&t_empty[buf], (uint32_t)(((g >> 1) - 1) & 1)))) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          ot_pairs<0, 0>(tmem + (uint32_t)buf * kOtBufCols, a0, sw128_desc(smem_u32(Bs + st * kOtBChunk)), idesc);
+        if (elect_one()) {
+          ot_pairs<0, 0>(tmem + (uint32_t)buf * kOtBufCols, a0, b_desc0 + (uint64_t)(st * (kOtBChunk >> 4)), idesc);
           umma_commit(&t_full[buf]);
           umma_commit(&b_empty[st]);
+          if (c == kOtChunks - 1) umma_commit(&a_empty[ab]);
         }
-        if (!ok) break;
-        umma_commit(&a_empty[ab]);
       }
-      if (!ok) atomicExch(&fail, 1);
-      // every table copy issued has landed and every MMA issued has finished
-      // before shared and tensor memory are released
-      for (int64_t gq = g; gq < issued; ++gq)
-        if (!mbar_wait(&b_full[gq % kOtBStages], (uint32_t)((gq / kOtBStages) & 1))) atomicExch(&fail, 1);
-      umma_commit(&mma_done);
-      if (!mbar_wait(&mma_done, 0)) atomicExch(&fail, 1);
-    }
+      return true;
+    };
+    for (int64_t it = 0; it < ntile && ok; it += 2)
+      ok = tile(a_desc0, 0, it) && (it + 1 >= ntile || tile(a_desc0 + (uint64_t)(kOtABytes >> 4), 1, it + 1));
+    if (!ok) atomicExch(&fail, 1);
+    // every table copy issued has landed and every MMA issued has finished
+    // before shared and tensor memory are released
+    for (int64_t gq = g; gq < issued; ++gq)
+      if (!mbar_wait_warp(&b_full[gq % kOtBStages], (uint32_t)((gq / kOtBStages) & 1))) atomicExch(&fail, 1);
+    if (elect_one()) umma_commit(&mma_done);
+    if (!mbar_wait_warp(&mma_done, 0)) atomicExch(&fail, 1);
   } else {
     // ------------------------------------------------------------ drain
     const int q = warp & 3;          // tensor-memory lane quarter
