@@ -184,6 +184,29 @@ __device__ __forceinline__ void ot_dft8_fix(long long (&x)[16]) {
   t = x[7]; x[7] = x[13]; x[13] = t;
 }
 
+// Sums of squares of the fixed-point X (|X| < 2^60.6; its lowest bit, below the
+// fixed point's own few units of error, is dropped): with X = A 2^32 + 2 b, b in
+// [-2^30, 2^30), X^2 = A^2 2^64 + A b 2^34 + b^2 4, each part summed exactly by one
+// 32 x 32 + 64-bit multiply-add (|A| < 2^28.7; eight squares stay below 2^63).
+// GB300 issues FP64 at 2 lanes a clock and SM, so a conversion and an FP64 FMA for
+// every value kept the FP64 pipe 76% busy and were what the top level waited
+// for; here the FP64 work is one value per bin and drain thread.
+struct OtSquares {
+  unsigned long long hh = 0, ll = 0;
+  long long hl = 0;
+  __device__ __forceinline__ void add(long long x) {
+    const uint32_t lo = (uint32_t)x;
+    const int A = (int)(x >> 32) + (int)(lo >> 31);
+    const int b = (int)lo >> 1;
+    hh += (unsigned long long)((long long)A * A);
+    hl += (long long)A * b;
+    ll += (unsigned long long)((long long)b * b);
+  }
+  __device__ __forceinline__ double value() const {
+    return fma(__ull2double_rn(hh), 0x1p64, fma(__ll2double_rn(hl), 0x1p34, 4.0 * __ull2double_rn(ll)));
+  }
+};
+
 // the largest exponent field among the values, as the scale exponent t with
 // |x| < 2^t; zero or subnormal only: 0 (their digits are zero)
 __device__ __forceinline__ int ot_scale_exp(int emax) {
@@ -331,6 +354,19 @@ struct OzTopArgs {
   double pscale;   // 1 / N^2
 };
 
+// The top level's drain keeps three 64-bit sums per bin in registers: 104 a
+// thread there, 64 in the producer and MMA warps (96 each at launch).
+template <int MODE, bool FEWER>
+__device__ __forceinline__ void ot_reg_share() {
+  static_assert(128 * 64 + (kOtThreads - 128) * 104 <= kOtThreads * 96, "the shares lie within the launch's registers");
+  if constexpr (MODE == 1) {
+    if constexpr (FEWER)
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    else
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+  }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
   pdl_begin();
@@ -387,6 +423,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
 
   if (warp < 3) {
     // ------------------------------------------------------------ producers
+    ot_reg_share<MODE, true>();
     // item u < 256 of a tile: half u & 1 (complex values 8 (u & 1) .. + 7) of
     // pencil u >> 1; items u and u ^ 1 run in adjacent lanes of one round
     int it = 0;
@@ -404,24 +441,26 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         const int64_t j = t * kOtRows + p;
         const bool have = j < a.npencils;  // rows past a partial tile's pencils: zero digits
         const double2* src = a.seeds + (have ? ((a.seed_rk + (j << a.seed_sh)) << 4) + 8 * half : 0);
-        double2 z[kOtD / 2];
         int emax = 0;
 #pragma unroll
         for (int k = 0; k < kOtD / 2; ++k) {
-          z[k] = have ? __ldg(src + k) : make_double2(0.0, 0.0);
-          emax = max(emax, (int)((__double_as_longlong(z[k].x) >> 52) & 0x7ff));
-          emax = max(emax, (int)((__double_as_longlong(z[k].y) >> 52) & 0x7ff));
+          const double2 z = have ? __ldg(src + k) : make_double2(0.0, 0.0);
+          emax = max(emax, (int)((__double_as_longlong(z.x) >> 52) & 0x7ff));
+          emax = max(emax, (int)((__double_as_longlong(z.y) >> 52) & 0x7ff));
         }
         emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
         const int tau = ot_scale_exp(emax);
-        // digit s of reals 4 g .. 4 g + 3 (two complex values) -> the half g & 1
-        // of chunk (s & 1) 4 + (g >> 1) of slab s >> 1
-#pragma unroll
+        // digit s of reals 4 g .. 4 g + 3 (two complex values, read again: they are
+        // in the L1 cache, and 32 registers less) -> the half g & 1 of chunk
+        // (s & 1) 4 + (g >> 1) of slab s >> 1
+#pragma unroll 1
         for (int gg = 0; gg < 4; ++gg) {
           const int g = 4 * half + gg;
+          const double2 z0 = have ? __ldg(src + 2 * gg) : make_double2(0.0, 0.0);
+          const double2 z1 = have ? __ldg(src + 2 * gg + 1) : make_double2(0.0, 0.0);
           uint32_t wa[kOtS], wb[kOtS];
-          ot_digit_pairs(z[2 * gg].x, z[2 * gg].y, tau, wa);
-          ot_digit_pairs(z[2 * gg + 1].x, z[2 * gg + 1].y, tau, wb);
+          ot_digit_pairs(z0.x, z0.y, tau, wa);
+          ot_digit_pairs(z1.x, z1.y, tau, wb);
 #pragma unroll
           for (int s = 0; s < kOtS; ++s)
             *reinterpret_cast<uint2*>(At + (s >> 1) * kOtSlabA + sw128_offset(p, (s & 1) * 4 + (g >> 1)) +
@@ -454,6 +493,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
     // tile and the two digit buffers are unrolled, so that every descriptor is a
     // constant away from a loop invariant (an MMA issues in 42 clocks, the read
     // rate of its operands, instead of about 100).
+    ot_reg_share<MODE, true>();
     const uint32_t idesc = make_idesc<kTcBF16, 32>();
     const uint64_t a_desc0 = sw128_desc(smem_u32(As)), b_desc0 = sw128_desc(smem_u32(Bs));
     const int64_t first = a.tile_begin + blockIdx.x;
@@ -510,6 +550,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
     if (!mbar_wait_warp(&mma_done, 0)) atomicExch(&fail, 1);
   } else {
     // ------------------------------------------------------------ drain
+    ot_reg_share<MODE, false>();
     const int q = warp & 3;          // tensor-memory lane quarter
     const int k = (warp - 4) >> 2;   // 0 .. 3
     const int h = k & 1;             // column i = 2 c + h of chunk c
@@ -532,9 +573,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
       // X in units of 2^(tau + sigma - 52) (the fixed point below)
       const int e2 = tauS[tb * kOtRows + row] - 22;
       const int64_t jt = t * kOtRows + row;  // local pencil index
-      double acc[kOtL];
-#pragma unroll
-      for (int y = 0; y < kOtL; ++y) acc[y] = 0.0;
+      OtSquares sq2[kOtL];
       for (int c = par; c < kOtChunks; c += 2, ++uses) {
         got = mbar_wait(&t_full[par], uses & 1);
         got = __all_sync(0xffffffffu, got && !*vfail) != 0;
@@ -574,9 +613,9 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
           }
         } else {
 #pragma unroll
-          for (int y = 0; y < kOtL; ++y) {
-            const double re = __ll2double_rn(x[2 * y]), im = __ll2double_rn(x[2 * y + 1]);
-            acc[y] = fma(re, re, fma(im, im, acc[y]));  // in units of 2^(2 e2)
+          for (int y = 0; y < kOtL; ++y) {  // in units of 2^(2 e2)
+            sq2[y].add(x[2 * y]);
+            sq2[y].add(x[2 * y + 1]);
           }
         }
       }
@@ -587,6 +626,9 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
       // the four partial sums of a bin meet in tensor memory: warps k = 1 .. 3
       // of a lane quarter store theirs in columns 448 + 16 (k - 1), warp 0 adds
       const uint32_t sqc = lane_base + kOtSqCol;
+      double acc[kOtL];
+#pragma unroll
+      for (int y = 0; y < kOtL; ++y) acc[y] = sq2[y].value();
       if (k != 0) {
         got = it < 1 || mbar_wait(&sq_empty, (it - 1) & 1);
         if (!__all_sync(0xffffffffu, got && !*vfail)) {
