@@ -202,10 +202,31 @@ struct OtSquares {
     hl += (long long)A * b;
     ll += (unsigned long long)((long long)b * b);
   }
+  // the sum as a double, by integer operations: all drain warps reach this at the
+  // end of a tile, and five FP64 operations a bin there took 10,000 clocks of the
+  // SM during which no accumulator was read
   __device__ __forceinline__ double value() const {
-    return fma(__ull2double_rn(hh), 0x1p64, fma(__ll2double_rn(hl), 0x1p34, 4.0 * __ull2double_rn(ll)));
+    const unsigned long long mid = (unsigned long long)hl << 34, low = ll << 2;
+    const unsigned long long lo = low + mid;
+    const unsigned long long hi = hh + (unsigned long long)(hl >> 30) + (ll >> 62) + (lo < low ? 1 : 0);
+    const unsigned long long top = hi ? hi : lo;
+    if (top == 0) return 0.0;
+    const int n = __clzll((long long)top);
+    const unsigned long long frac = (hi && n) ? (hi << n) | (lo >> (64 - n)) : top << n;  // leading bit at 63
+    const unsigned long long exp = (unsigned long long)(1023 + 63 + (hi ? 64 : 0) - n - 1);  // less the leading one
+    return __longlong_as_double((long long)((exp << 52) + (frac >> 11) + ((frac >> 10) & 1)));
   }
 };
+
+// better() for a bin v >= 0 (or NaN, which is never better): nonnegative doubles
+// order as their bits, off the FP64 pipe
+__device__ __forceinline__ void ot_better(double& best, int64_t& besty, double v, int64_t y) {
+  const long long bv = __double_as_longlong(v), bb = __double_as_longlong(best);
+  if (bv >= 0 && bv <= 0x7ff0000000000000LL && (bb < 0 || bv > bb || (bv == bb && y < besty))) {
+    best = v;
+    besty = y;
+  }
+}
 
 // the largest exponent field among the values, as the scale exponent t with
 // |x| < 2^t; zero or subnormal only: 0 (their digits are zero)
@@ -666,16 +687,19 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         const double f = a.pscale * ldexp(1.0, e2) * ldexp(1.0, e2);  // the units and 1 / N^2
         const int64_t j = jt;
         if (j < a.npencils) {
+          // outcome of bin y: y0 + y ystep; P y summed as y0 sum(P) + ystep sum(y P)
+          const int64_t y0 = a.rk + (j << a.sh), ystep = int64_t(1) << (lna + a.sh);
+          double s0 = 0.0, s1 = 0.0;
 #pragma unroll
           for (int y = 0; y < kOtL; ++y) {
             const double pv = acc[y] * f;
-            const int64_t yl = j + ((int64_t)y << lna);
-            a.hist[yl] = pv;
-            const int64_t yy = a.rk + (yl << a.sh);
-            better(best, besty, pv, yy);
-            wsum = fma(pv, (double)yy, wsum);
-            psum += pv;
+            a.hist[j + ((int64_t)y << lna)] = pv;
+            ot_better(best, besty, pv, y0 + y * ystep);
+            s0 += pv;
+            s1 = fma(pv, (double)y, s1);
           }
+          wsum = fma(s0, (double)y0, fma(s1, (double)ystep, wsum));
+          psum += s0;
         }
       }
     }
