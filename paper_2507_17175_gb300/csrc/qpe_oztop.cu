@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
   int4* twS = reinterpret_cast<int4*>(Bs + kOtBStages * kOtBChunk);  // [2][128][7] twiddles in Q61, split at bit 31
   int* tauS = reinterpret_cast<int*>(twS + 2 * kOtRows * (kOtL - 1));  // [2][128]
   __shared__ uint64_t a_full[2], a_empty[2], tw_empty[2], b_full[kOtBStages], b_empty[kOtBStages], t_full[2],
-      t_empty[2], sq_full, sq_empty, mma_done;
+      t_empty[2], sq_full[4], sq_empty[4], mma_done;
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
   __shared__ Partial sp[4];
@@ -419,8 +419,10 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
       mbar_init(&t_full[b], 1);
       mbar_init(&t_empty[b], 8);  // the drain warps of the buffer's chunks, two per lane quarter
     }
-    mbar_init(&sq_full, 12);
-    mbar_init(&sq_empty, 4);
+    for (int b = 0; b < 4; ++b) {  // one pair per lane quarter
+      mbar_init(&sq_full[b], 3);
+      mbar_init(&sq_empty[b], 1);
+    }
     mbar_init(&mma_done, 1);
     fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -456,6 +458,12 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         break;
       }
       if (*vfail) break;
+      // the next tile's rows (consecutive unless sharded) into L2 meanwhile
+      if (threadIdx.x == 0 && a.seed_sh == 0 && (t + gridDim.x + 1) * kOtRows <= a.npencils && t + gridDim.x < a.tile_end)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                         a.seeds + ((a.seed_rk + (t + gridDim.x) * kOtRows) << 4)),
+                     "r"((uint32_t)(kOtRows * kOtD * sizeof(double2)))
+                     : "memory");
       unsigned char* At = As + tb * kOtABytes;
       for (int u = threadIdx.x; u < 2 * kOtRows; u += kOtProducers) {
         const int p = u >> 1, half = u & 1;
@@ -490,12 +498,23 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         {  // the twiddles w_N^(m_b y_a): m_b = 1 .. 4 by half 0 (with the scale), 5 .. 7 by half 1
           const int64_t ya = a.rk + (j << a.sh);
           int4* tw = twS + (tb * kOtRows + p) * (kOtL - 1);
-          const int m0 = half == 0 ? 1 : 5, m1 = half == 0 ? 5 : kOtL;
-          for (int m = m0; m < m1; ++m) {
+          const int m0 = half == 0 ? 1 : 5;
+          // the table loads together: one after another their latencies were most
+          // of a producer's time
+          double2 wl[4], wh[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int m = m0 + i < kOtL ? m0 + i : kOtL - 1;
             const int64_t ex = (((int64_t)m * ya) & lvl_mask) << lvl_shift;
-            const double2 w = ot_cmul(__ldg(a.tw_lo + (ex & tw_mask)), __ldg(a.tw_hi + (ex >> a.htw)));
+            wl[i] = __ldg(a.tw_lo + (ex & tw_mask));
+            wh[i] = __ldg(a.tw_hi + (ex >> a.htw));
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (m0 + i >= kOtL) break;
+            const double2 w = ot_cmul(wl[i], wh[i]);
             const long long qr = ot_fixed(w.x, -6), qi = ot_fixed(w.y, -6);  // round(w 2^61)
-            tw[m - 1] =
+            tw[m0 + i - 1] =
                 make_int4((int)(qr >> 31), (int)(qr & 0x7fffffff), (int)(qi >> 31), (int)(qi & 0x7fffffff));
           }
           if (half == 0) tauS[tb * kOtRows + p] = tau + sigma - 30;
@@ -651,7 +670,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
 #pragma unroll
       for (int y = 0; y < kOtL; ++y) acc[y] = sq2[y].value();
       if (k != 0) {
-        got = it < 1 || mbar_wait(&sq_empty, (it - 1) & 1);
+        got = it < 1 || mbar_wait(&sq_empty[q], (it - 1) & 1);
         if (!__all_sync(0xffffffffu, got && !*vfail)) {
           ok = false;
           break;
@@ -666,9 +685,9 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         tmem_st16(sqc + (uint32_t)(16 * (k - 1)), w);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sq_full);
+        if (lane == 0) mbar_arrive(&sq_full[q]);
       } else {
-        got = mbar_wait(&sq_full, it & 1);
+        got = mbar_wait(&sq_full[q], it & 1);
         if (!__all_sync(0xffffffffu, got && !*vfail)) {
           ok = false;
           break;
@@ -683,7 +702,7 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sq_empty);
+        if (lane == 0) mbar_arrive(&sq_empty[q]);
         const double f = a.pscale * ldexp(1.0, e2) * ldexp(1.0, e2);  // the units and 1 / N^2
         const int64_t j = jt;
         if (j < a.npencils) {
