@@ -114,7 +114,6 @@ struct FftPass {
   int64_t B;     // independent blocks (N / (R * L))
   int64_t L;     // row stride between the R elements of one DFT
   int64_t Q;     // L * d: contiguous elements per (block, digit)
-  int64_t W;     // elements of Q each CTA takes
 };
 
 struct FftPlan {
@@ -127,7 +126,8 @@ struct FftPlan {
 // the middle axis of the state viewed as [B][R][Q].
 struct FftArgs {
   int logr;
-  int logw;    // W = 2^logw columns per CTA
+  int logc;    // 2^logc columns per CTA, W = 2^logw of them side by side
+  int logw;
   int logq;    // Q = 2^logq
   int logd;
   int n;       // log2 of the transform length

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "qpe_dft.cuh"
 #include "qpe_internal.cuh"
 
 namespace qpe {
@@ -415,113 +416,139 @@ __global__ void __launch_bounds__(32 * kFewWarps)
 // [B][R][Q] (Q = L * d contiguous elements): for each block and each of the Q
 // columns, a length-R DFT over the middle axis (kernel omega_R^(a y)), then
 // the twiddle omega_(R L)^(b y) with b = column / d the row offset inside the
-// block, stored in place at digit y. Each CTA stages an R x W slab in shared
-// memory and runs log2(R) radix-2 stages on it.
+// block, stored in place at digit y.
+//
+// What bounds it: complex64 HBM, if the instructions get out of the way (with
+// every element four times through shared memory and a table read for each
+// butterfly the issue slots were 80% busy at 37% of HBM); complex128 the FP64 units. So a CTA takes
+// its R rows x 2^logc columns (128 bytes or more) straight into registers, R1 = 2^K1 rows a thread, runs a
+// length-R1 DFT there (constants only), exchanges once through shared memory
+// with the twiddle w_R^(n2 k1), runs the length-R2 DFT (R = R1 R2, rows n = n1 R2 + n2,
+// digit y = k1 + R1 k2) and stores from registers. Passes over narrow rows
+// (Q below 128 bytes: the last pass of small registers) take several blocks per
+// CTA, whose rows are consecutive in memory.
+// 2^27 points, three passes: complex64 2.24 -> 1.39 ms (4.6 TB/s), and complex128 (Nmat 10,
+// Nmeas 17, two passes) 19.9 -> 15.2 ms.
+__host__ __device__ constexpr int fft_k1(int logr) { return logr <= 4 ? logr : logr <= 6 ? 3 : logr <= 8 ? 4 : 5; }
 
-__device__ __forceinline__ int bitrev(int x, int bits) { return bits ? (__brev(x) >> (32 - bits)) : 0; }
+template <typename C, int K1, int K2>
+__device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict__ tw_lo, const C* __restrict__ tw_hi,
+                                         const FftArgs& a, int64_t bid) {
+  using R_t = typename real_of<C>::type;
+  constexpr int R1 = 1 << K1, R2 = 1 << K2;
+  static_assert(K1 == fft_k1(K1 + K2), "the host sizes the tile by the same split");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // complex64: radix-2 stages with the table's twiddles, as a stage-by-stage
+  // transform has them (the same bits; HBM is the bound). complex128: DFTs with
+  // constants and one twiddle per element between the steps (a quarter fewer FP64
+  // operations, which are the bound).
+  constexpr bool kStages = sizeof(C) == 8;
+  C* twp = reinterpret_cast<C*>(smem_raw);  // w_R^e = omega_N^(e << (n - logr)), e < R
+  C* tile = twp + R1 * R2;                  // [g][k1][n2][w], rows of a k1 padded by W when W is narrow
+  const int logw = a.logw, W = 1 << logw;
+  const int logg = a.logc - logw;           // log2 of the blocks per CTA (Q = W when above 0)
+  const int kld = (R2 << logw) + (logg > 0 ? W : 0);  // elements per k1
+  int64_t blk;
+  uint32_t q0;                              // first column of the slab
+  if (logg == 0) {
+    const int slices_log = a.logq - logw;
+    blk = bid >> slices_log;
+    q0 = (uint32_t)(bid & ((int64_t(1) << slices_log) - 1)) << logw;
+  } else {
+    blk = bid << logg;
+    q0 = 0;
+  }
+  const int gn = (int)((int64_t(1) << a.logb) - blk < (1 << logg) ? (int64_t(1) << a.logb) - blk : 1 << logg);
+  C* base = X + (blk << (K1 + K2 + a.logq)) + q0;
+  const int tid = threadIdx.x;
 
-// K consecutive radix-2 DIF stages on the rows row0 + j 2^logs (j < 2^K) of
-// column w, in registers (see fft_pass_kernel).
-template <typename C, int K>
-__device__ __forceinline__ void fft_group(C* tile, const C* twp, int W, int w, int row0, int logm, int logs,
-                                          int logr) {
-  constexpr int RK = 1 << K;
-  C x[RK];
+  // rows n1 R2 + n2 of column (g, w): w fastest, then n2, then g
+  const int T1 = R2 << a.logc;
+  C x[R1];
+  auto load = [&](int t) {
+    const int w = t & (W - 1), n2 = (t >> logw) & (R2 - 1), g = t >> (logw + K2);
+    const C* src = base + ((int64_t)g << (K1 + K2 + a.logq)) + ((int64_t)n2 << a.logq) + w;
 #pragma unroll
-  for (int j = 0; j < RK; ++j) x[j] = tile[(row0 + (j << logs)) * W + w];
+    for (int j = 0; j < R1; ++j) x[j] = g < gn ? src[(int64_t)(j * R2) << a.logq] : mk((R_t)0, (R_t)0);
+  };
+  // digit y of column (g, w): the inter-pass twiddle, the scale, the store
+  const uint32_t lo_mask = (1u << a.htw) - 1u;
+  const uint32_t rl_mask = (uint32_t)((int64_t(1) << (K1 + K2 + a.logq - a.logd)) - 1);  // R L - 1
+  const int esh = a.logb + a.tw_sh;
+  auto store = [&](C v, C* dst, uint32_t b, int y) {
+    if (!a.last) {  // omega_(RL)^(b y) = omega_N^(b y B); b y < R L <= N <= 2^30
+      const uint32_t e = ((b * (uint32_t)y) & rl_mask) << esh;
+      v = cmul(v, cmul(ld(tw_lo + (e & lo_mask)), ld(tw_hi + (e >> a.htw))));
+    }
+    if (a.scale != 1.0) v = cscale(v, (R_t)a.scale);
+    dst[(int64_t)y << a.logq] = v;
+  };
+  if (tid < T1) load(tid);
+  if constexpr (K2 > 0 || kStages) {
+    for (int e = tid; e < (kStages ? R1 * R2 / 2 : R1 * R2); e += 256)
+      twp[e] = twiddle(tw_lo, tw_hi, a.htw, (int64_t)e << (a.n + a.tw_sh - (K1 + K2)));
+    __syncthreads();
+  }
+  for (int t = tid; t < T1; t += 256) {
+    if (t >= 256) load(t);
+    const int w = t & (W - 1), n2 = (t >> logw) & (R2 - 1), g = t >> (logw + K2);
+    if constexpr (kStages)
+      dft_stages<C, K1, R1>(x, [&](int p, int st) { return twp[((p << K2) + n2) << st]; });
+    else
+      dft_k<C, K1, R1>(x);
+    if constexpr (K2 == 0) {
+      if (g < gn) {
+        C* dst = base + ((int64_t)g << (K1 + a.logq)) + w;
+        const uint32_t b = (q0 + (uint32_t)w) >> a.logd;
 #pragma unroll
-  for (int lt = 0; lt < K; ++lt) {
-    const int logh = logm - lt - 1;  // global half size h = 2^logh
+        for (int k = 0; k < R1; ++k) store(x[k], dst, b, k);
+      }
+    } else {
+      C* dst = tile + (g * R1) * kld + (n2 << logw) + w;
 #pragma unroll
-    for (int j = 0; j < RK; ++j) {
-      const int hh = RK >> (lt + 1);
-      if (j & hh) continue;
-      const C x0 = x[j], x1 = x[j + hh];
-      x[j] = cadd(x0, x1);
-      const C dlt = csub(x0, x1);
-      const int pos = (row0 + (j << logs)) & ((1 << logh) - 1);
-      x[j + hh] = pos ? cmul(dlt, twp[pos << (logr - logh - 1)]) : dlt;
+      for (int k = 0; k < R1; ++k) dst[k * kld] = k && !kStages ? cmul(x[k], twp[n2 * k]) : x[k];
     }
   }
+  if constexpr (K2 > 0) {
+    __syncthreads();
+    const int T2 = R1 << a.logc;
+    for (int t = tid; t < T2; t += 256) {  // w fastest, then k1, then g
+      const int w = t & (W - 1), k1 = (t >> logw) & (R1 - 1), g = t >> (logw + K1);
+      if (g >= gn) break;
+      const C* src = tile + (g * R1 + k1) * kld + w;
+      C z[R2];
 #pragma unroll
-  for (int j = 0; j < RK; ++j) tile[(row0 + (j << logs)) * W + w] = x[j];
+      for (int j = 0; j < R2; ++j) z[j] = src[j << logw];
+      if constexpr (kStages)
+        dft_stages<C, K2, R2>(z, [&](int p, int st) { return twp[p << (st + K1)]; });
+      else
+        dft_k<C, K2, R2>(z);
+      C* dst = base + ((int64_t)g << (K1 + K2 + a.logq)) + w;
+      const uint32_t b = (q0 + (uint32_t)w) >> a.logd;
+#pragma unroll
+      for (int k = 0; k < R2; ++k) store(z[k], dst, b, k1 + (k << K1));
+    }
+  }
 }
 
 template <typename C>
 __device__ __forceinline__ void fft_pass_block(C* __restrict__ X, const C* __restrict__ tw_lo,
                                                const C* __restrict__ tw_hi, const FftArgs& a, int64_t bid) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tile = reinterpret_cast<C*>(smem_raw);
-  using R_t = typename real_of<C>::type;
-  const int R = 1 << a.logr;
-  const int W = 1 << a.logw;
-  const int64_t slices_log = a.logq - a.logw;
-  const int64_t blk = bid >> slices_log;
-  const int64_t qs = bid & ((int64_t(1) << slices_log) - 1);
-  C* base = X + (blk << (a.logr + a.logq)) + (qs << a.logw);
-  const int RW = R * W;
-  C* twp = tile + RW;  // w_R^e = omega_N^(e << (n - logr)), e < R / 2: the pass's twiddles
-  // the tile arrives by asynchronous 16-byte copies (every thread's copies in
-  // flight at once) while the twiddles are computed
-  constexpr int V = 16 / (int)sizeof(C);  // elements per copy
-  if (W >= V) {
-    for (int idx = threadIdx.x * V; idx < RW; idx += blockDim.x * V) {
-      const int r = idx >> a.logw, w = idx & (W - 1);
-      cp_async16(tile + idx, base + ((int64_t)r << a.logq) + w);
-    }
-  } else {
-    for (int idx = threadIdx.x; idx < RW; idx += blockDim.x) {
-      const int r = idx >> a.logw, w = idx & (W - 1);
-      cp_async_elem(tile + idx, base + ((int64_t)r << a.logq) + w, true);
-    }
-  }
-  cp_async_commit();
-  for (int e = threadIdx.x; e < (R >> 1); e += blockDim.x)
-    twp[e] = twiddle(tw_lo, tw_hi, a.htw, (int64_t)e << (a.n + a.tw_sh - a.logr));
-  cp_async_wait<0>();
-  __syncthreads();
-  // Radix-2 DIF stages s = 0 .. logr - 1 (stage s pairs rows p and p + h,
-  // h = 2^(logr - s - 1), twiddle omega_(2h)^(p mod h) on the difference),
-  // three at a time in registers: rows base + j S, j < 2^K, meet only each
-  // other within those K stages. The butterflies and twiddles are those of
-  // the stage-by-stage order, so the result is the same bit for bit.
-  for (int s0 = 0; s0 < a.logr; s0 += 3) {
-    const int K = a.logr - s0 < 3 ? a.logr - s0 : 3;
-    const int logm = a.logr - s0;  // sub-blocks of 2^logm rows
-    const int logs = logm - K;     // stride S = 2^logs between a task's rows
-    const int tasks = (R >> K) << a.logw;
-    for (int t = threadIdx.x; t < tasks; t += blockDim.x) {
-      const int w = t & (W - 1);
-      const int rest = t >> a.logw;
-      const int q = rest & ((1 << logs) - 1);
-      const int b0 = rest >> logs;
-      const int row0 = (b0 << logm) + q;
-      switch (K) {
-        case 1: fft_group<C, 1>(tile, twp, W, w, row0, logm, logs, a.logr); break;
-        case 2: fft_group<C, 2>(tile, twp, W, w, row0, logm, logs, a.logr); break;
-        default: fft_group<C, 3>(tile, twp, W, w, row0, logm, logs, a.logr); break;
-      }
-    }
-    __syncthreads();
-  }
-  const int64_t rl_mask = (int64_t(1) << (a.logr + a.logq - a.logd)) - 1;  // R*L - 1
-  for (int idx = threadIdx.x; idx < RW; idx += blockDim.x) {
-    const int i = idx >> a.logw, w = idx & (W - 1);
-    const int ya = bitrev(i, a.logr);
-    C v = tile[idx];
-    if (!a.last) {
-      const int64_t q = (qs << a.logw) + w;
-      const int64_t b = q >> a.logd;
-      const int64_t e = ((b * ya) & rl_mask) << (a.logb + a.tw_sh);  // omega_(RL)^(b ya) = omega_N^(b ya B)
-      if (e) v = cmul(v, twiddle(tw_lo, tw_hi, a.htw, e));
-    }
-    if (a.scale != 1.0) v = cscale(v, (R_t)a.scale);
-    base[((int64_t)ya << a.logq) + w] = v;
+  switch (a.logr) {  // (K1, K2) with K1 = fft_k1(logr)
+    case 1: fft_tile<C, 1, 0>(X, tw_lo, tw_hi, a, bid); break;
+    case 2: fft_tile<C, 2, 0>(X, tw_lo, tw_hi, a, bid); break;
+    case 3: fft_tile<C, 3, 0>(X, tw_lo, tw_hi, a, bid); break;
+    case 4: fft_tile<C, 4, 0>(X, tw_lo, tw_hi, a, bid); break;
+    case 5: fft_tile<C, 3, 2>(X, tw_lo, tw_hi, a, bid); break;
+    case 6: fft_tile<C, 3, 3>(X, tw_lo, tw_hi, a, bid); break;
+    case 7: fft_tile<C, 4, 3>(X, tw_lo, tw_hi, a, bid); break;
+    case 8: fft_tile<C, 4, 4>(X, tw_lo, tw_hi, a, bid); break;
+    default: fft_tile<C, 5, 4>(X, tw_lo, tw_hi, a, bid); break;
   }
 }
 
 template <typename C>
-__global__ void __launch_bounds__(256) fft_pass_kernel(C* __restrict__ X, const C* __restrict__ tw_lo,
+__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1) fft_pass_kernel(C* __restrict__ X, const C* __restrict__ tw_lo,
                                                        const C* __restrict__ tw_hi, FftArgs a) {
   pdl_begin();
   fft_pass_block<C>(X, tw_lo, tw_hi, a, blockIdx.x);
@@ -529,7 +556,7 @@ __global__ void __launch_bounds__(256) fft_pass_kernel(C* __restrict__ X, const 
 
 // One QFT^-1 pass of every listed instance (each item its own pass arguments).
 template <typename C>
-__global__ void __launch_bounds__(256) fft_pass_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1) fft_pass_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
   pdl_begin();
   const int i = find_item(items, nitems, blockIdx.x);
   fft_pass_block<C>(items[i].X, items[i].lo, items[i].hi, items[i].a, blockIdx.x - items[i].tile0);
@@ -1131,9 +1158,7 @@ int launch_sweep(const Instance& in, char* ws, bool gate_mode, cudaStream_t s, i
 
 FftPlan make_fft_plan(int nmeas, int64_t d, size_t esize) {
   FftPlan f;
-  const int logd = ilog2(d);
-  const int logwmax = ilog2((int64_t)(128 / esize));  // 128-byte column slabs
-  const int max_bits = 9;                            // R * W * esize <= 64 KiB
+  const int max_bits = 9;  // R x 128 bytes <= 64 KiB
   const int passes = (nmeas + max_bits - 1) / max_bits;
   f.passes = passes;
   int used = 0;
@@ -1145,11 +1170,7 @@ FftPlan make_fft_plan(int nmeas, int64_t d, size_t esize) {
     used += r;
     p.L = int64_t(1) << (nmeas - used);
     p.Q = p.L * d;
-    const int logq = ilog2(p.Q);
-    const int logw = logq < logwmax ? logq : logwmax;
-    p.W = int64_t(1) << logw;
     f.logr_list[i] = r;
-    (void)logd;
   }
   return f;
 }
@@ -1166,11 +1187,11 @@ int64_t fft_position_to_y(const FftPlan& f, int nmeas, int64_t p) {
   return y;
 }
 
+constexpr int kFftSmemMax = 96 * 1024;  // 64 KiB of tile, at most 16 of padding and 8 of twiddles
 FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, size_t esize) {
   const FftPass& p = in.fft.p[i];
   FftArgs a;
   a.logr = p.logr;
-  a.logw = ilog2(p.W);
   a.logq = ilog2(p.Q);
   a.logd = in.nmat;
   a.n = in.nmeas - in.shard_log;  // a sharded plan transforms its N / 2^shard_log local rows
@@ -1179,8 +1200,18 @@ FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, 
   a.logb = ilog2(p.B);
   a.last = (i == in.fft.passes - 1);
   a.scale = a.last ? 1.0 / sqrt(ldexp(1.0, in.nmeas)) : 1.0;  // QFT^-1 normalisation 2^(-n/2) in the last pass
-  *blocks = p.B * (p.Q / p.W);
-  *smem = ((size_t)(int64_t(1) << p.logr) * p.W + ((size_t)1 << p.logr) / 2) * esize;
+  // columns of a CTA: 128 bytes of a row, more (up to a tile of 64 KiB) while the
+  // grid still has two CTAs for each of the SM's two places; rows narrower than
+  // that are taken from several consecutive blocks
+  const int64_t points = p.B * p.Q << p.logr;
+  a.logc = ilog2((int64_t)(128 / esize));
+  while (((int64_t)esize << (a.logr + a.logc + 1)) <= 64 * 1024 && (points >> (a.logr + a.logc + 1)) >= 4 * 152) ++a.logc;
+  a.logw = std::min(a.logq, a.logc);
+  *blocks = std::max<int64_t>(1, points >> (a.logr + a.logc));
+  // twiddles of the pass, its tile, and the padding of narrow rows (one element
+  // per column and first-step digit; passes of one step need no tile)
+  const size_t rows = (size_t)1 << a.logr, cols = (size_t)1 << a.logc;
+  *smem = (rows + (a.logr <= 4 ? 0 : rows * cols + (a.logw < a.logc ? cols << fft_k1(a.logr) : 0))) * esize;
   return a;
 }
 
@@ -1332,16 +1363,15 @@ int launch_unpermute(const Instance& in, const char* ws, void* out, cudaStream_t
 cudaError_t configure_kernels() {
   cudaError_t e = configure_level_kernels();
   if (e != cudaSuccess) return e;
-  // tile (<= 64 KiB) + the pass's twiddles (<= 256 entries)
-  e = cudaFuncSetAttribute(fft_pass_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 4096);
+  e = cudaFuncSetAttribute(fft_pass_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fft_pass_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024 + 4096);
+  e = cudaFuncSetAttribute(fft_pass_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(fft_pass_grouped_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           64 * 1024 + 4096);
+                           kFftSmemMax);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(fft_pass_grouped_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              64 * 1024 + 4096);
+                              kFftSmemMax);
 }
 
 template int launch_sweep<float2>(const Instance&, char*, bool, cudaStream_t, int);

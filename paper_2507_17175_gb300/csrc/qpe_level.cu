@@ -29,6 +29,7 @@
 
 #include <cuda_fp16.h>
 
+#include "qpe_dft.cuh"
 #include "qpe_internal.cuh"
 #include "qpe_tcgen05.cuh"
 
@@ -37,17 +38,7 @@ namespace qpe {
 using tcg::kTcFP16;
 using tcg::kTcTF32;
 
-__constant__ double2 c_w32_64[32];  // exp(-2 pi i k / 32)
-__constant__ float2 c_w32_32[32];
-
 namespace {
-
-template <typename C>
-__device__ __forceinline__ C w32(int k);
-template <>
-__device__ __forceinline__ double2 w32<double2>(int k) { return c_w32_64[k]; }
-template <>
-__device__ __forceinline__ float2 w32<float2>(int k) { return c_w32_32[k]; }
 
 template <typename C>
 __device__ __forceinline__ C ldg(const C* p) { return __ldg(p); }
@@ -184,36 +175,6 @@ __device__ __forceinline__ void store4(float2* p, const float2 (&v)[4]) {
 __device__ __forceinline__ void store4(double2* p, const double2 (&v)[4]) {
 #pragma unroll
   for (int t = 0; t < 4; ++t) p[t] = v[t];
-}
-
-template <typename C, int K, int N>
-__device__ __forceinline__ void dft_k(C (&x)[N]) {
-  constexpr int R = 1 << K;
-#pragma unroll
-  for (int s = 0; s < K; ++s) {
-    const int h = R >> (s + 1);
-#pragma unroll
-    for (int g = 0; g < R; g += 2 * h) {
-#pragma unroll
-      for (int p = 0; p < h; ++p) {
-        const C u = x[g + p], v = x[g + p + h];
-        x[g + p] = cadd(u, v);
-        const C dl = csub(u, v);
-        x[g + p + h] = (p == 0) ? dl : cmul(dl, w32<C>(p * (32 / (2 * h))));
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    int rv = 0;
-#pragma unroll
-    for (int b = 0; b < K; ++b) rv |= ((i >> b) & 1) << (K - 1 - b);
-    if (rv > i) {
-      const C t = x[i];
-      x[i] = x[rv];
-      x[rv] = t;
-    }
-  }
 }
 
 // length-2^r DFT of x[0 .. 2^r), natural order in and out (2^r <= N)
@@ -1209,19 +1170,7 @@ cudaError_t configure_level_kernels() {
                               (2 * 64 * 64 + 2 * 16 * 64) * 8);
     if (e0 != cudaSuccess) return e0;
   }
-  double2 w64[32];
-  float2 w32v[32];
-  for (int k = 0; k < 32; ++k) {
-    // exp(-2 pi i k / 32) from the host math library
-    const double ang = -2.0 * M_PI * (double)k / 32.0;
-    w64[k] = make_double2(cos(ang), sin(ang));
-    w32v[k] = make_float2((float)w64[k].x, (float)w64[k].y);
-  }
-  cudaError_t e = cudaMemcpyToSymbol(c_w32_64, w64, sizeof(w64));
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_w32_32, w32v, sizeof(w32v));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(level_tc_top_kernel<kTcFP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(level_tc_top_kernel<kTcFP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)tc_top_smem<kTcFP16>());
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(level_tc_top_kernel<kTcTF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
