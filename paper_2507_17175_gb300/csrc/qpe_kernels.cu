@@ -228,6 +228,33 @@ __device__ __forceinline__ void rows_times_pt_tile(C* __restrict__ S, const C* _
                                                    Rows rows, int64_t bx, int by) {
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int TCOLS = BN / TN;
+  if constexpr (BN <= 4) {
+    // d = 2, 4: a thread owns a row (16-byte loads and stores, P from the L1 cache,
+    // the same order of additions), HBM is the bound: d = 4, 2^25 rows complex64 by
+    // doubling 568 -> 260 us
+    static_assert(NT == BM, "a thread per row");
+    const int64_t lr = bx * BM + threadIdx.x;
+    if (lr >= M) return;
+    constexpr int V = 16 / (int)sizeof(C);  // elements per load
+    union Row {
+      C e[BN];
+      float4 v[BN / V];
+    } in, out;
+    const float4* src = reinterpret_cast<const float4*>(S + rows.in(lr) * BN);
+#pragma unroll
+    for (int q = 0; q < BN / V; ++q) in.v[q] = src[q];
+#pragma unroll
+    for (int j = 0; j < BN; ++j) {
+      C acc = mk((typename real_of<C>::type)0, (typename real_of<C>::type)0);
+#pragma unroll
+      for (int k = 0; k < BN; ++k) cfma(acc, in.e[k], ld(P + j * BN + k));
+      out.e[j] = acc;
+    }
+    float4* dst = reinterpret_cast<float4*>(S + rows.out(lr) * BN);
+#pragma unroll
+    for (int q = 0; q < BN / V; ++q) dst[q] = out.v[q];
+    return;
+  }
   __shared__ C As[BK][BM + 1];
   __shared__ C Bs[BK][BN + 1];
   const int tid = threadIdx.x;
@@ -431,11 +458,16 @@ __global__ void __launch_bounds__(32 * kFewWarps)
 // Nmeas 17, two passes) 19.9 -> 15.2 ms.
 __host__ __device__ constexpr int fft_k1(int logr) { return logr <= 4 ? logr : logr <= 6 ? 3 : logr <= 8 ? 4 : 5; }
 
+// complex128 takes up to 32 points in 128 registers a thread: CTAs of half the
+// threads, so that two of them share an SM and one computes while the other loads
+template <typename C>
+constexpr int kFftThreads = sizeof(C) == 8 ? 256 : 128;
+
 template <typename C, int K1, int K2>
 __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict__ tw_lo, const C* __restrict__ tw_hi,
                                          const FftArgs& a, int64_t bid) {
   using R_t = typename real_of<C>::type;
-  constexpr int R1 = 1 << K1, R2 = 1 << K2;
+  constexpr int R1 = 1 << K1, R2 = 1 << K2, NT = kFftThreads<C>;
   static_assert(K1 == fft_k1(K1 + K2), "the host sizes the tile by the same split");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // complex64: radix-2 stages with the table's twiddles, as a stage-by-stage
@@ -485,12 +517,12 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
   };
   if (tid < T1) load(tid);
   if constexpr (K2 > 0 || kStages) {
-    for (int e = tid; e < (kStages ? R1 * R2 / 2 : R1 * R2); e += 256)
+    for (int e = tid; e < (kStages ? R1 * R2 / 2 : R1 * R2); e += NT)
       twp[e] = twiddle(tw_lo, tw_hi, a.htw, (int64_t)e << (a.n + a.tw_sh - (K1 + K2)));
     __syncthreads();
   }
-  for (int t = tid; t < T1; t += 256) {
-    if (t >= 256) load(t);
+  for (int t = tid; t < T1; t += NT) {
+    if (t >= NT) load(t);
     const int w = t & (W - 1), n2 = (t >> logw) & (R2 - 1), g = t >> (logw + K2);
     if constexpr (kStages)
       dft_stages<C, K1, R1>(x, [&](int p, int st) { return twp[((p << K2) + n2) << st]; });
@@ -512,7 +544,7 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
   if constexpr (K2 > 0) {
     __syncthreads();
     const int T2 = R1 << a.logc;
-    for (int t = tid; t < T2; t += 256) {  // w fastest, then k1, then g
+    for (int t = tid; t < T2; t += NT) {  // w fastest, then k1, then g
       const int w = t & (W - 1), k1 = (t >> logw) & (R1 - 1), g = t >> (logw + K1);
       if (g >= gn) break;
       const C* src = tile + (g * R1 + k1) * kld + w;
@@ -548,7 +580,7 @@ __device__ __forceinline__ void fft_pass_block(C* __restrict__ X, const C* __res
 }
 
 template <typename C>
-__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1) fft_pass_kernel(C* __restrict__ X, const C* __restrict__ tw_lo,
+__global__ void __launch_bounds__(kFftThreads<C>, 2) fft_pass_kernel(C* __restrict__ X, const C* __restrict__ tw_lo,
                                                        const C* __restrict__ tw_hi, FftArgs a) {
   pdl_begin();
   fft_pass_block<C>(X, tw_lo, tw_hi, a, blockIdx.x);
@@ -556,7 +588,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1) fft_pass_kernel(C
 
 // One QFT^-1 pass of every listed instance (each item its own pass arguments).
 template <typename C>
-__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 2 : 1) fft_pass_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
+__global__ void __launch_bounds__(kFftThreads<C>, 2) fft_pass_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
   pdl_begin();
   const int i = find_item(items, nitems, blockIdx.x);
   fft_pass_block<C>(items[i].X, items[i].lo, items[i].hi, items[i].a, blockIdx.x - items[i].tile0);
@@ -633,16 +665,29 @@ __device__ __forceinline__ void reduce_block(const C* __restrict__ X, double* __
       const int kc = (int)(t % kc_count);
       const int64_t mbits = t / kc_count;
       const int64_t ybase = (mbits << 5);
-      // reads: k fastest across the threads (consecutive positions)
+      // reads: k fastest across the threads (consecutive positions); the position
+      // of y = ybase + ylo + (k << shift_hi) is ybase's with ylo in the top digit
+      // and k in the lowest
+      const int64_t pbase = y_to_pos(g, n, ybase) + (int64_t)kc * K;
+      const int top = n - g.logr[0];
       for (int e = threadIdx.x; e < 32 * K; e += 256) {
-        const int k = e % K, ylo = e / K;
-        const int64_t y = ybase + ylo + (int64_t(kc * K + k) << shift_hi);
-        const C* row = X + (y_to_pos(g, n, y) << logd);
+        const int k = e & (K - 1), ylo = e / K;
+        const C* row = X + ((pbase + ((int64_t)ylo << top) + k) << logd);
         if constexpr (sizeof(C) == 8) {
           float f = 0.f;
-          for (int q = 0; q < d; ++q) {
-            const C v = __ldg(row + q);
+          if (d == 2) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(row));
             f = fmaf(v.x, v.x, fmaf(v.y, v.y, f));
+            f = fmaf(v.z, v.z, fmaf(v.w, v.w, f));
+          } else {  // d = 4, 8
+            for (int q = 0; q < d; q += 4) {
+              const float4 v = __ldg(reinterpret_cast<const float4*>(row + q));
+              const float4 u = __ldg(reinterpret_cast<const float4*>(row + q + 2));
+              f = fmaf(v.x, v.x, fmaf(v.y, v.y, f));
+              f = fmaf(v.z, v.z, fmaf(v.w, v.w, f));
+              f = fmaf(u.x, u.x, fmaf(u.y, u.y, f));
+              f = fmaf(u.z, u.z, fmaf(u.w, u.w, f));
+            }
           }
           tile_f[ylo * 129 + k] = f * (float)scale;  // scale is a power of two
         } else {
@@ -666,7 +711,7 @@ __device__ __forceinline__ void reduce_block(const C* __restrict__ X, double* __
             best_f = v;
             by = y;
           }
-          float t1 = v * (float)y - wcomp_f;
+          float t1 = v * __int2float_rn((int)y) - wcomp_f;  // y < 2^30
           float t2 = wsum_f + t1;
           wcomp_f = (t2 - wsum_f) - t1;
           wsum_f = t2;
@@ -867,9 +912,50 @@ __global__ void __launch_bounds__(256) finalize_kernel(const Partial* __restrict
   }
 }
 
+// Rows from digit-reversed positions to natural order, in 16-byte pieces (VR =
+// log2 of the pieces per row). Rows of at most 64 bytes with two digits or more
+// go through shared memory in tiles of 32 consecutive y times K values of y's
+// highest digit, which is the position's lowest: read as runs of K rows, written as
+// runs of 32 (2^25 rows of 32 bytes: 780 -> 420 us; a row at a time leaves every
+// 32-byte sector in its own DRAM burst).
+constexpr int kUnpermuteTile = 2048;  // 16-byte pieces
+__global__ void __launch_bounds__(256) unpermute_kernel(const float4* __restrict__ X, float4* __restrict__ out,
+                                                        int64_t N, int vr, int n, Digits g) {
+  pdl_begin();
+  __shared__ float4 tile[kUnpermuteTile + 32];
+  const int lb = g.count >= 2 ? g.logr[g.count - 1] : 0;
+  if (vr <= 2 && g.count >= 2 && g.logr[0] >= 5) {
+    const int kcap = 11 - 5 - vr;                 // log2 of the rows of a run
+    const int lk = lb < kcap ? lb : kcap, K = 1 << lk;
+    const int shift_hi = n - lb, top = n - g.logr[0];
+    const int kc_log = lb - lk;
+    const int64_t ntiles = int64_t(1) << (n - 5 - lk);
+    const int run = K << vr;                      // pieces of a run, padded by one row of pieces
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const int64_t kc = t & ((int64_t(1) << kc_log) - 1), ybase = (t >> kc_log) << 5;
+      const float4* src = X + ((y_to_pos(g, n, ybase) + (kc << lk)) << vr);
+      for (int e = threadIdx.x; e < 32 * run; e += 256) {
+        const int ylo = e >> (lk + vr), q = e & (run - 1);
+        tile[ylo * (run + 1) + q] = __ldcs(src + ((int64_t)ylo << (top + vr)) + q);
+      }
+      __syncthreads();
+      float4* dst = out + (((ybase + (kc << (lk + shift_hi)))) << vr);
+      for (int e = threadIdx.x; e < 32 * run; e += 256) {
+        const int v = e & ((1 << vr) - 1), ylo = (e >> vr) & 31, k = e >> (vr + 5);
+        __stcs(dst + ((int64_t)k << (shift_hi + vr)) + (ylo << vr) + v, tile[ylo * (run + 1) + (k << vr) + v]);
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  const int64_t total = N << vr, mask = (int64_t(1) << vr) - 1;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = X[(y_to_pos(g, n, i >> vr) << vr) | (i & mask)];
+}
+// the same element by element, for an output on an 8-byte boundary
 template <typename C>
-__global__ void unpermute_kernel(const C* __restrict__ X, C* __restrict__ out, int64_t N, int logd, int n,
-                                 Digits g) {
+__global__ void unpermute_elements_kernel(const C* __restrict__ X, C* __restrict__ out, int64_t N, int logd, int n,
+                                          Digits g) {
   pdl_begin();
   const int64_t total = N << logd;
   const int64_t dmask = (int64_t(1) << logd) - 1;
@@ -1225,7 +1311,7 @@ int launch_fft(const Instance& in, char* ws, cudaStream_t s) {
     int64_t blocks = 0;
     size_t smem = 0;
     const FftArgs a = fft_pass_args(in, i, &blocks, &smem, sizeof(C));
-    if (launch_k(fft_pass_kernel<C>, dim3((unsigned)blocks), dim3(256), smem, s, X, lo, hi, a) != cudaSuccess)
+    if (launch_k(fft_pass_kernel<C>, dim3((unsigned)blocks), dim3(kFftThreads<C>), smem, s, X, lo, hi, a) != cudaSuccess)
       return -1;
     ++launches;
   }
@@ -1286,7 +1372,7 @@ int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, 
 template <typename C>
 int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, cudaStream_t s) {
   if (nitems <= 0) return 0;
-  return launch_k(fft_pass_grouped_kernel<C>, dim3((unsigned)blocks), dim3(256), smem, s, items, nitems) ==
+  return launch_k(fft_pass_grouped_kernel<C>, dim3((unsigned)blocks), dim3(kFftThreads<C>), smem, s, items, nitems) ==
                  cudaSuccess
              ? 1
              : -1;
@@ -1352,8 +1438,15 @@ int launch_finalize(const Instance& in, char* ws, int count, cudaStream_t s) {
 template <typename C>
 int launch_unpermute(const Instance& in, const char* ws, void* out, cudaStream_t s) {
   const Digits g = digits_of(in.fft);
-  return launch_k(unpermute_kernel<C>, dim3(grid_for(in.N * in.d, 256)), dim3(256), 0, s,
-                  reinterpret_cast<const C*>(ws + in.off_state), reinterpret_cast<C*>(out), in.N, in.nmat, in.nmeas,
+  if (reinterpret_cast<uintptr_t>(out) % 16 != 0)
+    return launch_k(unpermute_elements_kernel<C>, dim3(grid_for(in.N * in.d, 256)), dim3(256), 0, s,
+                    reinterpret_cast<const C*>(ws + in.off_state), reinterpret_cast<C*>(out), in.N, in.nmat, in.nmeas,
+                    g) == cudaSuccess
+               ? 1
+               : -1;
+  const int vr = in.nmat - (sizeof(C) == 8 ? 1 : 0);  // a row is 2^vr pieces of 16 bytes
+  return launch_k(unpermute_kernel, dim3(grid_for(in.N << vr, 8 * 256)), dim3(256), 0, s,
+                  reinterpret_cast<const float4*>(ws + in.off_state), reinterpret_cast<float4*>(out), in.N, vr, in.nmeas,
                   g) == cudaSuccess
              ? 1
              : -1;
