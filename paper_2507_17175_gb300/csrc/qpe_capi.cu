@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -29,6 +30,12 @@ namespace {
 constexpr int kMaxNmat = 12;
 constexpr int kMaxNmeas = 30;
 constexpr size_t kAlign = 256;
+
+// the readout and the device error word as they lie in the workspace
+struct ReadBack {
+  qpe::Scalars s;
+  int32_t err;
+};
 
 size_t align_up(size_t v) { return (v + kAlign - 1) & ~(kAlign - 1); }
 
@@ -63,7 +70,7 @@ size_t layout_instance(Instance& in, int prec, uint32_t flags, size_t base, bool
   in.fused = in.nmat <= QPE_MAX_FUSED_NMAT && !(flags & (QPE_FLAG_PLAIN | QPE_FLAG_GATE_SWEEP)) &&
              (!is_tc(prec) || batched || in.nmat <= 4);
   in.keep_state = (flags & QPE_FLAG_KEEP_STATE) != 0;
-  if (in.nmat <= QPE_MAX_FUSED_NMAT) in.levels = qpe::make_levels(in.nmeas, in.nmat, elem_size(prec), 0);
+  if (in.nmat <= QPE_MAX_FUSED_NMAT) in.levels = qpe::make_levels(in.nmeas, in.nmat, elem_size(prec), true);
   // the fused schedule never materialises the N x d state unless asked to keep
   // it; a sharded plan keeps (and histograms) only its own N / 2^shard_log rows
   in.state_bytes = (size_t)(N >> in.shard_log) * d * elem_size(prec);
@@ -77,8 +84,9 @@ size_t layout_instance(Instance& in, int prec, uint32_t flags, size_t base, bool
   in.off_tw_lo32 = take(nlo * 8);
   in.off_tw_hi32 = take(nhi * 8);
   in.off_partials = take(sizeof(qpe::Partial) * qpe::kReduceBlocks);
-  in.off_scalars = take(sizeof(qpe::Scalars));
-  in.off_err = take(sizeof(int));
+  // the error word right behind the readout: one copy reads both back
+  in.off_scalars = take(sizeof(ReadBack));
+  in.off_err = in.off_scalars + offsetof(ReadBack, err);
   if (is_tc(prec) && !in.fused) in.off_tcsplit = take(qpe::tc_split_bytes(prec, in.nmat, in.nmeas));
   // sharded plain schedule: all-to-all buffers of the local transform
   in.shard_plain = !in.fused && in.shard_log > 0;
@@ -1050,7 +1058,7 @@ qpe_status qpe_plan_shard(const qpe_plan_desc* desc, int32_t rank, int32_t world
   } else {
     // the fused form partitions the outcomes; the top level must have at
     // least `world` pencils
-    const std::vector<qpe::Level> lv = qpe::make_levels(desc->nmeas, desc->nmat, elem_size(desc->prec), 0);
+    const std::vector<qpe::Level> lv = qpe::make_levels(desc->nmeas, desc->nmat, elem_size(desc->prec), false);
     if (lv.empty() || lv[0].logna < sh) return QPE_ERR_UNSUPPORTED;
   }
   qpe_plan_s* p = new (std::nothrow) qpe_plan_s();
@@ -1347,14 +1355,12 @@ qpe_status qpe_sync(qpe_plan_t p) {
   if (e != cudaSuccess) return cuda_fail(p, e, "cudaStreamSynchronize");
   for (const Instance& in : p->inst) {
     if (!in.loaded) continue;
-    int derr = 0;
-    e = cudaMemcpy(&derr, p->ws + in.off_err, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(p, e, "read error word");
-    if (derr) return fail(p, (qpe_status)derr, err_word_message(derr));
+    ReadBack rb{};
+    e = cudaMemcpy(&rb, p->ws + in.off_scalars, sizeof(rb), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(p, e, "read the readout and the error word");
+    if (rb.err) return fail(p, (qpe_status)rb.err, err_word_message(rb.err));
     if (in.state_stage != QPE_STAGE_REDUCE) continue;
-    qpe::Scalars s;
-    e = cudaMemcpy(&s, p->ws + in.off_scalars, sizeof(s), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(p, e, "read readout scalars");
+    const qpe::Scalars& s = rb.s;
     if (s.err) return fail(p, (qpe_status)s.err, "device flagged a non-finite histogram");
   }
   return QPE_OK;
@@ -1372,12 +1378,13 @@ qpe_status qpe_probs(qpe_plan_t p, int32_t instance, double* probs, int64_t* arg
   if (probs && probs != in->host_hist)  // the host histogram buffer already holds the run's bins
     e = cudaMemcpyAsync(probs, p->ws + in->off_hist, (size_t)(in->N >> in->shard_log) * 8,
                         kind_from_device(ptr_is_device), p->stream);
-  qpe::Scalars s;
-  int derr = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&s, p->ws + in->off_scalars, sizeof(s), cudaMemcpyDeviceToHost, p->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&derr, p->ws + in->off_err, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
+  ReadBack rb{};
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&rb, p->ws + in->off_scalars, sizeof(rb), cudaMemcpyDeviceToHost, p->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
   if (e != cudaSuccess) return cuda_fail(p, e, "qpe_probs copy");
+  const qpe::Scalars& s = rb.s;
+  const int derr = rb.err;
   if (derr) return fail(p, (qpe_status)derr, err_word_message(derr));
   if (argmax) *argmax = s.argmax;
   if (phase_argmax) *phase_argmax = s.phase_argmax;

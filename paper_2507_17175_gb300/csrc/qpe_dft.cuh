@@ -63,8 +63,11 @@ __device__ __forceinline__ void dft_k(C (&x)[N]) {
 // The same by radix-2 decimation-in-frequency stages whose twiddles tw(p, s) =
 // w^(p 2^s) the caller supplies (stage s pairs points p and p + 2^(K - s - 1) of its
 // blocks): as the first K stages of a longer transform, or its last ones.
-template <typename C, int K, int N, typename Tw>
-__device__ __forceinline__ void dft_stages(C (&x)[N], Tw tw) {
+// The roundings of a butterfly's product are written out, so that they do not
+// depend on how the surrounding code is compiled.
+template <int K, int N, typename Tw>
+__device__ __forceinline__ void dft_stages(float2 (&x)[N], Tw tw) {
+  using C = float2;
   constexpr int R = 1 << K;
 #pragma unroll
   for (int s = 0; s < K; ++s) {
@@ -76,7 +79,8 @@ __device__ __forceinline__ void dft_stages(C (&x)[N], Tw tw) {
       for (int g = 0; g < R; g += 2 * h) {
         const C u = x[g + p], v = x[g + p + h];
         x[g + p] = cadd(u, v);
-        x[g + p + h] = cmul(csub(u, v), w);
+        const C dl = csub(u, v);
+        x[g + p + h] = mk(__fmaf_rn(dl.x, w.x, -__fmul_rn(dl.y, w.y)), __fmaf_rn(dl.y, w.x, __fmul_rn(dl.x, w.y)));
       }
     }
   }

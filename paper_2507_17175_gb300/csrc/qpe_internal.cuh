@@ -686,7 +686,7 @@ int64_t oz_gate_tiles(const Instance& in, int j);
 int launch_oz_gate_grouped(const OzItem* pits, const RowSliceItem* rits, const OzItem* gits, const GateRound& R,
                            cudaStream_t s);
 int level_max_bits(int logd, size_t esize, size_t smem_cap);
-std::vector<Level> make_levels(int nmeas, int logd, size_t esize, int rtop);
+std::vector<Level> make_levels(int nmeas, int logd, size_t esize, bool balanced);
 // a level of a sharded plan computes only this rank's outcomes when it has at
 // least 2^shard_log pencils; smaller (deeper) levels are computed whole
 bool level_sharded(const Instance& in, int li);

@@ -525,7 +525,7 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
     if (t >= NT) load(t);
     const int w = t & (W - 1), n2 = (t >> logw) & (R2 - 1), g = t >> (logw + K2);
     if constexpr (kStages)
-      dft_stages<C, K1, R1>(x, [&](int p, int st) { return twp[((p << K2) + n2) << st]; });
+      dft_stages<K1, R1>(x, [&](int p, int st) { return twp[((p << K2) + n2) << st]; });
     else
       dft_k<C, K1, R1>(x);
     if constexpr (K2 == 0) {
@@ -552,7 +552,7 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
 #pragma unroll
       for (int j = 0; j < R2; ++j) z[j] = src[j << logw];
       if constexpr (kStages)
-        dft_stages<C, K2, R2>(z, [&](int p, int st) { return twp[p << (st + K1)]; });
+        dft_stages<K2, R2>(z, [&](int p, int st) { return twp[p << (st + K1)]; });
       else
         dft_k<C, K2, R2>(z);
       C* dst = base + ((int64_t)g << (K1 + K2 + a.logq)) + w;

@@ -27,6 +27,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include <cuda_fp16.h>
 
 #include "qpe_dft.cuh"
@@ -1121,15 +1123,20 @@ bool level_sharded(const Instance& in, int li) {
   return in.shard_log > 0 && in.levels[li].logna >= in.shard_log;
 }
 
-std::vector<Level> make_levels(int nmeas, int logd, size_t esize, int rtop) {
-  const int rmax = level_max_bits(logd, esize, kLevelSmemCap);
+// Levels of r <= rmax bits, the top one first. At most 256 outcomes are a matter of
+// latency: a level of five bits is one pencil or two whose 32-point FP64 DFTs and
+// five-factor table rows run on a few lanes of one SM, so `balanced` splits them into
+// equal levels of at most four bits (Nmat 2, Nmeas 6 FP64: top level 61 -> 15 us).
+std::vector<Level> make_levels(int nmeas, int logd, size_t esize, bool balanced) {
+  int rmax = level_max_bits(logd, esize, kLevelSmemCap);
+  if (balanced && nmeas <= 8 && rmax > 4) {
+    const int count = (nmeas + 3) / 4;
+    rmax = (nmeas + count - 1) / count;
+  }
   std::vector<Level> lv;
   int remaining = nmeas, off = 0;
-  bool top = true;
   while (remaining > 0) {
-    int r = top ? (rtop > 0 ? rtop : rmax) : rmax;
-    if (r > rmax) r = rmax;
-    if (r > remaining) r = remaining;
+    const int r = std::min(rmax, remaining);
     Level L{};
     L.off = off;
     L.r = r;
@@ -1137,7 +1144,6 @@ std::vector<Level> make_levels(int nmeas, int logd, size_t esize, int rtop) {
     lv.push_back(L);
     off += r;
     remaining -= r;
-    top = false;
   }
   return lv;
 }
