@@ -423,8 +423,8 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
       oz.sb0 = O.sblocks;
       oz.e0 = O.elems;
       oz.tile0 = O.tiles;
-      O.sblocks += 2 * in.d;
-      O.elems += in.d * in.d;
+      O.sblocks += qpe::oz_scale_ctas(in.d);
+      O.elems += qpe::oz_slice_tiles(in.d);
       O.tiles += qpe::oz_square_tiles(in);
       bm.oz_items.push_back(oz);
     }
@@ -629,8 +629,8 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
             if (!qpe::oz_gate_items(in, ws, j, rowbuf, &pit, &rit, &git)) throw std::runtime_error("tensor map");
             pit.sb0 = G.sblocks;
             pit.e0 = G.elems;
-            G.sblocks += 2 * in.d;
-            G.elems += in.d * in.d;
+            G.sblocks += qpe::oz_scale_ctas(in.d);
+            G.elems += qpe::oz_slice_tiles(in.d);
             rit.tile0 = G.rows;
             G.rows += int64_t(1) << j;
             git.tile0 = G.tiles;

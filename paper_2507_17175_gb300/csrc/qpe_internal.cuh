@@ -497,8 +497,8 @@ struct OzArgs {
   int64_t row_out = 0;
 };
 // One instance's squaring step in a grouped launch: the digit slices' tensor
-// maps, P_k, the slice buffers, and the item's first scale block, first slice
-// element and first GEMM CTA in the launches' numbering.
+// maps, P_k, the slice buffers (B null: not wanted), and the item's first scale CTA, first slice
+// tile and first GEMM CTA in the launches' numbering.
 struct OzItem {
   CUtensorMap mA, mB;
   OzArgs a;
@@ -645,6 +645,8 @@ size_t oz_square_bytes(int nmat);
 // CTAs, and the three launches (scales, slices, GEMM) for all items of a step
 bool oz_square_item(const Instance& in, char* ws, int k, bool want_c64, OzItem* it);
 int64_t oz_square_tiles(const Instance& in);
+int64_t oz_scale_ctas(int64_t d);
+int64_t oz_slice_tiles(int64_t d);
 int launch_square_oz_grouped(const OzItem* items, int nitems, int64_t sblocks, int64_t elems, int64_t tiles,
                              cudaStream_t s);
 int launch_square_oz(const Instance& in, char* ws, int k, bool want_c64, cudaStream_t s);

@@ -270,30 +270,9 @@ __device__ __forceinline__ void ot_digits(double x, int t, int (&dg)[kOtS]) {
 // bf16 bits of a small integer (|v| <= 256: exact in the upper half of the float)
 __device__ __forceinline__ uint32_t ot_bf16(int v) { return __float_as_uint((float)v) >> 16; }
 
-// The balanced digits of F = round(x 2^(55 - t)) (|F| <= 2^55) from the plain
-// base-256 digits of F + B, B = 128 sum_(s<7) 2^(8 s) (0 <= F + B < 2^57):
-// digit s is byte 6 - s of F + B minus 128 (the top one takes bits 48..56).
-// Each becomes a float by the magic-number form 2^23 + d minus 2^23 + 128
-// (exact), whose upper half is its bf16; w[s] packs digit s of x0 (low half)
-// and x1 (high half).
-constexpr unsigned long long kOtBias = 0x80808080808080ull;
-__device__ __forceinline__ float ot_byte_digit(uint32_t word, uint32_t sel) {
-  return __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u | sel)) - 8388736.0f;
-}
+// The balanced digits of round(x 2^(55 - t)) of two values, packed in pairs
 __device__ __forceinline__ void ot_digit_pairs(double x0, double x1, int t, uint32_t (&w)[kOtS]) {
-  const unsigned long long u0 = (unsigned long long)ot_fixed(x0, t) + kOtBias;
-  const unsigned long long u1 = (unsigned long long)ot_fixed(x1, t) + kOtBias;
-  const uint32_t l0 = (uint32_t)u0, h0 = (uint32_t)(u0 >> 32), l1 = (uint32_t)u1, h1 = (uint32_t)(u1 >> 32);
-  const float t0 = __uint_as_float(0x4B000000u | (h0 >> 16)) - 8388736.0f;
-  const float t1 = __uint_as_float(0x4B000000u | (h1 >> 16)) - 8388736.0f;
-  w[0] = __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x7632);
-#pragma unroll
-  for (int s = 1; s < kOtS; ++s) {
-    const int byte = 6 - s;
-    const float f0 = ot_byte_digit(byte >= 4 ? h0 : l0, (uint32_t)(byte & 3));
-    const float f1 = ot_byte_digit(byte >= 4 ? h1 : l1, (uint32_t)(byte & 3));
-    w[s] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-  }
+  digit_words(ot_fixed(x0, t), ot_fixed(x1, t), w);
 }
 
 __device__ __forceinline__ double2 ot_cmul(double2 a, double2 b) {

@@ -480,46 +480,67 @@ __global__ void split_grouped_kernel(const TcSplitItem* __restrict__ items, int 
 // the integer sum of the pairs of weight w over K. The pairs with w <= 6 are
 // formed (28 bf16 products); the rest lie below 2^-53 of 2^(tau + sigma) K.
 constexpr int kOzS = 7;       // digits per operand entry
-constexpr int kOzBeta = 8;    // bits per digit
 
 __device__ __forceinline__ double pow2d(int e) {  // 2^e for -1022 <= e <= 1023
   return __longlong_as_double((long long)(1023 + e) << 52);
 }
 
-// exponent t with 0 < |x| < 2^t for the largest |x| of a row or column; tiny
-// or zero lines get a floor (their digits are all zero)
-__device__ __forceinline__ int oz_exponent(double mx) {
-  if (!(mx > 0x1p-900)) return -900;
-  const int eb = (int)((__double_as_longlong(mx) >> 52) & 0x7ff) - 1023;
-  return eb + 1;
+// Scales and digits by integer operations on the bits (GB300's FP64 units would
+// take 2 lanes a clock and SM for the comparisons and conversions), each entry of
+// P read once per pass in runs, each digit plane written in 4-byte pairs. At
+// d = 2048 the three launches of a squaring's slicing (two passes over P by
+// columns, FP64 conversions, 2-byte stores) took 380 us; two take 110 us (the
+// bytes alone: 60).
+//
+// Exponent field of the largest |x| of a row or column -> t with |x| < 2^t; tiny or zero
+// lines get a floor (their digits are all zero).
+__device__ __forceinline__ int oz_exponent(int emax) { return emax - 1022 < -900 ? -900 : emax - 1022; }
+__device__ __forceinline__ int oz_field(double2 p) {
+  return max((__double2hiint(p.x) >> 20) & 0x7ff, (__double2hiint(p.y) >> 20) & 0x7ff);
+}
+
+// round(x 2^(55 - t)), halves to even, for |x| < 2^t
+__device__ __forceinline__ long long oz_fixed(double x, int t) {
+  const long long b = __double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7ff), k = E - 1020 - t;  // x 2^(55 - t) = M 2^k, k <= 2
+  const long long M = (b & 0xfffffffffffffLL) | 0x10000000000000LL;
+  long long F = 0;
+  if (k >= 0)
+    F = k < 8 ? M << k : 0;  // (a non-finite line has set the error word)
+  else if (k > -54 && E > 0)
+    F = (M + ((1LL << (-k - 1)) - 1) + ((M >> -k) & 1)) >> -k;
+  return b < 0 ? -F : F;
 }
 
 // tau[i]: scale of rows i and i + d of E (from row i of P); sig[j]: of column
-// j of [Re P ; Im P]. A non-finite entry sets the error word.
+// j of [Re P ; Im P]. A non-finite entry sets the error word. CTAs 0 .. d / 8 - 1
+// take eight rows each (one per warp), the next d / 16 sixteen columns each.
 __device__ __forceinline__ void oz_scale_block(const double2* __restrict__ P, int d, int* __restrict__ tau,
                                                int* __restrict__ sig, int* __restrict__ err, int b) {
-  double mx = 0.0;
-  bool finite = true;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    const double2 p = b < d ? P[(int64_t)b * d + k] : P[(int64_t)k * d + (b - d)];
-    finite = finite && isfinite(p.x) && isfinite(p.y);
-    mx = fmax(mx, fmax(fabs(p.x), fabs(p.y)));
+  __shared__ int wm[8][16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int m = 0;
+  if (b < d / 8) {
+    const int r = b * 8 + warp;
+    const double2* row = P + (int64_t)r * d;
+#pragma unroll 4
+    for (int k = lane; k < d; k += 32) m = max(m, oz_field(__ldg(row + k)));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) tau[r] = oz_exponent(m);
+  } else {
+    const int c = (b - d / 8) * 16 + (lane & 15);
+#pragma unroll 8
+    for (int k = warp * 2 + (lane >> 4); k < d; k += 16) m = max(m, oz_field(__ldg(P + (int64_t)k * d + c)));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    if (lane < 16) wm[warp][lane] = m;
+    __syncthreads();
+    if (threadIdx.x < 16) {
+      for (int w = 1; w < 8; ++w) m = max(m, wm[w][lane]);
+      sig[c] = oz_exponent(m);
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  __shared__ double wm[8];
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = mx;
-  if (__syncthreads_or(!finite) && threadIdx.x == 0) atomicCAS(err, 0, (int)QPE_ERR_NUMERIC);
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, wm[w]);
-    mx = fmax(mx, wm[0]);
-    const int e = oz_exponent(mx);
-    if (b < d)
-      tau[b] = e;
-    else
-      sig[b - d] = e;
-  }
+  if (m == 0x7ff) atomicCAS(err, 0, (int)QPE_ERR_NUMERIC);
 }
-
 __global__ void __launch_bounds__(256) oz_scale_kernel(const double2* __restrict__ P, int d, int* __restrict__ tau,
                                                        int* __restrict__ sig, int* __restrict__ err) {
   pdl_begin();
@@ -527,103 +548,102 @@ __global__ void __launch_bounds__(256) oz_scale_kernel(const double2* __restrict
   pdl_trigger();
 }
 
-// balanced base-2^8 digits of x at scale 2^t, most significant first:
-// out[s * stride], s = 0 .. kOzS - 1
-__device__ __forceinline__ void oz_digits(double x, int t, __nv_bfloat16* out, int64_t stride) {
-  long long F = __double2ll_rn(x * pow2d(kOzS * kOzBeta - 1 - t));  // |F| < 2^55
+// The digits of a 32 x 32 tile of P: A[(s 2d + m) 2d + kk] of E's rows (2d x 2d) and,
+// when B is given, B[(s d + n) 2d + kk] of E[kk][n] (n < d); also the complex64 copy of P
+// when A32 is given.
+constexpr int kOzTile = 32;
+__device__ __forceinline__ void oz_slice_tile(const double2* __restrict__ P, int d, const int* __restrict__ tau,
+                                              const int* __restrict__ sig, __nv_bfloat16* __restrict__ A,
+                                              __nv_bfloat16* __restrict__ B, float2* __restrict__ A32, int t) {
+  __shared__ double2 T[kOzTile][kOzTile + 1];
+  const int per = d / kOzTile;
+  const int i0 = t / per * kOzTile, j0 = t % per * kOzTile;
+  for (int e = threadIdx.x; e < kOzTile * kOzTile; e += 256) {
+    const int r = e / kOzTile, c = e % kOzTile;
+    const int64_t at = (int64_t)(i0 + r) * d + j0 + c;
+    const double2 p = __ldg(P + at);
+    T[r][c] = p;
+    if (A32) A32[at] = make_float2((float)p.x, (float)p.y);
+  }
+  __syncthreads();
+  const int64_t d2 = 2 * (int64_t)d;
+  auto put = [](__nv_bfloat16* at, uint32_t v) { *reinterpret_cast<uint32_t*>(at) = v; };
+  for (int e = threadIdx.x; e < kOzTile * kOzTile / 2; e += 256) {
+    const int r = e / (kOzTile / 2), c = e % (kOzTile / 2) * 2;
+    const int ts = tau[i0 + r];
+    const double2 p = T[r][c], q = T[r][c + 1];
+    const long long px = oz_fixed(p.x, ts), qx = oz_fixed(q.x, ts), py = oz_fixed(p.y, ts), qy = oz_fixed(q.y, ts);
+    uint32_t re[kOzS], im[kOzS], mi[kOzS];
+    digit_words(px, qx, re);
+    digit_words(py, qy, im);
+    digit_words(-py, -qy, mi);
+    __nv_bfloat16* o = A + (int64_t)(i0 + r) * d2 + j0 + c;
 #pragma unroll
-  for (int s = kOzS - 1; s >= 1; --s) {
-    long long r = F & 255;
-    if (r >= 128) r -= 256;
-    out[(int64_t)s * stride] = __float2bfloat16_rn((float)r);
-    F = (F - r) / 256;
+    for (int s = 0; s < kOzS; ++s, o += d2 * d2) {
+      put(o, re[s]);               // E[i][j]     = Re
+      put(o + d * d2 + d, re[s]);  // E[i+d][j+d] = Re
+      put(o + d, mi[s]);           // E[i][j+d]   = -Im
+      put(o + d * d2, im[s]);      // E[i+d][j]   = Im
+    }
   }
-  out[0] = __float2bfloat16_rn((float)F);
-}
-
-// digits of E (rows 2d, K = 2d) per slice: A[(s 2d + m) 2d + kk]; also the
-// complex64 copy of P when A32 is given
-__device__ __forceinline__ void oz_slice_a_elem(const double2* __restrict__ P, int d, const int* __restrict__ tau,
-                                                __nv_bfloat16* __restrict__ A, float2* __restrict__ A32, int64_t e) {
-  const int64_t d2 = 2 * (int64_t)d, stride = d2 * d2;
-  {
-    const int64_t i = e / d, j = e - i * d;
-    const double2 p = P[e];
-    if (A32) A32[e] = make_float2((float)p.x, (float)p.y);
-    const int t = tau[i];
-    oz_digits(p.x, t, A + i * d2 + j, stride);             // E[i][j]     = Re
-    oz_digits(p.x, t, A + (i + d) * d2 + j + d, stride);   // E[i+d][j+d] = Re
-    oz_digits(-p.y, t, A + i * d2 + j + d, stride);        // E[i][j+d]   = -Im
-    oz_digits(p.y, t, A + (i + d) * d2 + j, stride);       // E[i+d][j]   = Im
+  if (!B) return;
+  for (int e = threadIdx.x; e < kOzTile * kOzTile / 2; e += 256) {
+    const int n = e / (kOzTile / 2), c = e % (kOzTile / 2) * 2;
+    const int ts = sig[j0 + n];
+    const double2 p = T[c][n], q = T[c + 1][n];
+    uint32_t re[kOzS], im[kOzS];
+    digit_words(oz_fixed(p.x, ts), oz_fixed(q.x, ts), re);
+    digit_words(oz_fixed(p.y, ts), oz_fixed(q.y, ts), im);
+    __nv_bfloat16* o = B + (int64_t)(j0 + n) * d2 + i0 + c;
+#pragma unroll
+    for (int s = 0; s < kOzS; ++s, o += d * d2) {
+      put(o, re[s]);      // E[kk][n]   = Re P[kk][n]
+      put(o + d, im[s]);  // E[kk+d][n] = Im P[kk][n]
+    }
   }
 }
-
-__global__ void __launch_bounds__(256) oz_slice_a_kernel(const double2* __restrict__ P, int d,
-                                                         const int* __restrict__ tau, __nv_bfloat16* __restrict__ A,
-                                                         float2* __restrict__ A32) {
+__global__ void __launch_bounds__(256) oz_slice_kernel(const double2* __restrict__ P, int d,
+                                                       const int* __restrict__ tau, const int* __restrict__ sig,
+                                                       __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
+                                                       float2* __restrict__ A32) {
   pdl_begin();
-  const int64_t dd = (int64_t)d * d;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < dd; e += (int64_t)gridDim.x * blockDim.x)
-    oz_slice_a_elem(P, d, tau, A, A32, e);
+  oz_slice_tile(P, d, tau, sig, A, B, A32, blockIdx.x);
   pdl_trigger();
 }
-
-// digits of B (rows d, K = 2d): B[(s d + n) 2d + kk] = digits of E[kk][n]
-__device__ __forceinline__ void oz_slice_b_elem(const double2* __restrict__ P, int d, const int* __restrict__ sig,
-                                                __nv_bfloat16* __restrict__ B, int64_t e) {
-  const int64_t d2 = 2 * (int64_t)d, stride = (int64_t)d * d2;
-  {
-    const int64_t n = e / d, kk = e - n * d;  // consecutive threads: consecutive kk (contiguous writes)
-    const double2 p = P[kk * d + n];
-    const int t = sig[n];
-    oz_digits(p.x, t, B + n * d2 + kk, stride);      // E[kk][n]   = Re P[kk][n]
-    oz_digits(p.y, t, B + n * d2 + kk + d, stride);  // E[kk+d][n] = Im P[kk][n]
-  }
-}
-
-__global__ void __launch_bounds__(256) oz_slice_b_kernel(const double2* __restrict__ P, int d,
-                                                         const int* __restrict__ sig, __nv_bfloat16* __restrict__ B) {
-  pdl_begin();
-  const int64_t dd = (int64_t)d * d;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < dd; e += (int64_t)gridDim.x * blockDim.x)
-    oz_slice_b_elem(P, d, sig, B, e);
-  pdl_trigger();
-}
-
 
 // Digits of state row r for a gate level: [Re S_r | Im S_r] (2d reals) at the
 // row's own scale tau[r], A[(s M + r) 2d + k]; the whole CTA takes part. A
 // non-finite entry sets the error word.
 __device__ __forceinline__ void oz_slice_row(const double2* __restrict__ S, int64_t M, int d, int* __restrict__ tau,
                                              __nv_bfloat16* __restrict__ A, int* __restrict__ err, int64_t r) {
-  __shared__ double wm[8];
-  __shared__ int t_s;
+  __shared__ int wm[8];
   const double2* row = S + r * d;
-  double mx = 0.0;
-  bool finite = true;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    const double2 p = row[k];
-    finite = finite && isfinite(p.x) && isfinite(p.y);
-    mx = fmax(mx, fmax(fabs(p.x), fabs(p.y)));
-  }
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = mx;
-  if (__syncthreads_or(!finite) && threadIdx.x == 0) atomicCAS(err, 0, (int)QPE_ERR_NUMERIC);
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, wm[w]);
-    t_s = oz_exponent(fmax(mx, wm[0]));
-    tau[r] = t_s;
-  }
+  int m = 0;
+  for (int k = threadIdx.x; k < d; k += 256) m = max(m, oz_field(row[k]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
   __syncthreads();
-  const int t = t_s;
-  const int64_t stride = M * 2 * (int64_t)d;
-  __nv_bfloat16* out = A + r * 2 * (int64_t)d;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    const double2 p = row[k];
-    oz_digits(p.x, t, out + k, stride);
-    oz_digits(p.y, t, out + d + k, stride);
+#pragma unroll
+  for (int w = 0; w < 8; ++w) m = max(m, wm[w]);
+  const int t = oz_exponent(m);
+  if (threadIdx.x == 0) {
+    tau[r] = t;
+    if (m == 0x7ff) atomicCAS(err, 0, (int)QPE_ERR_NUMERIC);
   }
-  __syncthreads();  // wm and t_s are reused by the next row
+  const int64_t stride = M * 2 * (int64_t)d;
+  for (int k = 2 * threadIdx.x; k < d; k += 512) {
+    const double2 p = row[k], q = row[k + 1];
+    uint32_t re[kOzS], im[kOzS];
+    digit_words(oz_fixed(p.x, t), oz_fixed(q.x, t), re);
+    digit_words(oz_fixed(p.y, t), oz_fixed(q.y, t), im);
+    __nv_bfloat16* o = A + r * 2 * (int64_t)d + k;
+#pragma unroll
+    for (int s = 0; s < kOzS; ++s, o += stride) {
+      *reinterpret_cast<uint32_t*>(o) = re[s];
+      *reinterpret_cast<uint32_t*>(o + d) = im[s];
+    }
+  }
+  __syncthreads();  // wm is reused by the next row
 }
 
 __global__ void __launch_bounds__(256) oz_slice_rows_kernel(const double2* __restrict__ S, int64_t M, int d,
@@ -987,7 +1007,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_square_kernel(const __grid_c
 // slices, then the digit-product GEMM with per-item tensor maps.
 __global__ void __launch_bounds__(256) oz_scale_grouped_kernel(const OzItem* __restrict__ items, int nitems) {
   pdl_begin();
-  int lo = 0, hi = nitems - 1;  // item whose scale blocks [sb0, sb0 + 2d) hold this CTA
+  int lo = 0, hi = nitems - 1;  // item whose scale CTAs, from sb0 on, hold this one
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (items[mid].sb0 <= (int64_t)blockIdx.x)
@@ -1001,23 +1021,19 @@ __global__ void __launch_bounds__(256) oz_scale_grouped_kernel(const OzItem* __r
   pdl_trigger();
 }
 
-__global__ void __launch_bounds__(256) oz_slice_grouped_kernel(const OzItem* __restrict__ items, int nitems,
-                                                               int64_t elems) {
+__global__ void __launch_bounds__(256) oz_slice_grouped_kernel(const OzItem* __restrict__ items, int nitems) {
   pdl_begin();
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < elems; e += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nitems - 1;  // item whose elements [e0, e0 + d^2) hold e
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (items[mid].e0 <= e)
-        lo = mid;
-      else
-        hi = mid - 1;
-    }
-    const OzItem& it = items[lo];
-    const int64_t le = e - it.e0;
-    oz_slice_a_elem(it.P, it.a.d, it.a.tau, static_cast<__nv_bfloat16*>(it.A), it.A32, le);
-    oz_slice_b_elem(it.P, it.a.d, it.a.sig, static_cast<__nv_bfloat16*>(it.B), le);
+  int lo = 0, hi = nitems - 1;  // item whose tiles, from e0 on, hold this CTA
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (items[mid].e0 <= (int64_t)blockIdx.x)
+      lo = mid;
+    else
+      hi = mid - 1;
   }
+  const OzItem& it = items[lo];
+  oz_slice_tile(it.P, it.a.d, it.a.tau, it.a.sig, static_cast<__nv_bfloat16*>(it.A),
+                static_cast<__nv_bfloat16*>(it.B), it.A32, (int)(blockIdx.x - it.e0));
   pdl_trigger();
 }
 
@@ -1100,6 +1116,10 @@ cudaError_t configure_tc_kernels() {
   return cudaFuncSetAttribute(oz_square_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem());
 }
 
+// CTAs of a squaring step's scale and slicing launches
+int64_t oz_scale_ctas(int64_t d) { return d / 8 + d / 16; }
+int64_t oz_slice_tiles(int64_t d) { return (d / kOzTile) * (d / kOzTile); }
+
 // Workspace of the tensor-core squaring: row / column scales and the digit
 // slices of E (kOzS x 2d x 2d) and of B (kOzS x d x 2d), bf16.
 size_t oz_square_bytes(int nmat) {
@@ -1121,12 +1141,10 @@ int launch_square_oz(const Instance& in, char* ws, int k, bool want_c64, cudaStr
   __nv_bfloat16* A = reinterpret_cast<__nv_bfloat16*>(base + ((2 * (size_t)d * sizeof(int) + 255) & ~size_t(255)));
   __nv_bfloat16* B = A + (size_t)kOzS * 4 * dd;
   int* err = reinterpret_cast<int*>(ws + in.off_err);
-  cudaError_t e = launch_k(oz_scale_kernel, dim3(2 * d), dim3(256), 0, s, P, d, tau, sig, err);
-  const unsigned eb = (unsigned)std::min<int64_t>((dd + 255) / 256, 152 * 16);
+  cudaError_t e = launch_k(oz_scale_kernel, dim3((unsigned)oz_scale_ctas(d)), dim3(256), 0, s, P, d, tau, sig, err);
   if (e == cudaSuccess)
-    e = launch_k(oz_slice_a_kernel, dim3(eb), dim3(256), 0, s, P, d, (const int*)tau, A,
-                 (P32 && k == 1) ? P32 : (float2*)nullptr);
-  if (e == cudaSuccess) e = launch_k(oz_slice_b_kernel, dim3(eb), dim3(256), 0, s, P, d, (const int*)sig, B);
+    e = launch_k(oz_slice_kernel, dim3((unsigned)oz_slice_tiles(d)), dim3(256), 0, s, P, d, (const int*)tau,
+                 (const int*)sig, A, B, (P32 && k == 1) ? P32 : (float2*)nullptr);
   if (e != cudaSuccess) return -1;
   CUtensorMap mA, mB;
   if (!make_map(&mA, A, kTcBF16, (int64_t)kOzS * 2 * d, 2 * (int64_t)d, kBM) ||
@@ -1135,7 +1153,7 @@ int launch_square_oz(const Instance& in, char* ws, int k, bool want_c64, cudaStr
   OzArgs a{tau, sig, C, P32 ? P32 + k * dd : nullptr, d, err};
   const unsigned grid = (unsigned)((2 * d / kBM) * (d / kOzBN));
   e = launch_k(oz_square_kernel, dim3(grid), dim3(kOzThreads), oz_smem(), s, mA, mB, a);
-  return e == cudaSuccess ? 4 : -1;
+  return e == cudaSuccess ? 3 : -1;
 }
 
 // Workspace of the FP64 gate levels on the tensor cores: the state rows'
@@ -1165,10 +1183,10 @@ int launch_oz_gate_level(const Instance& in, char* ws, int j, int pow_off, cudaS
   const int64_t Mmax = (in.N >> in.shard_log) / 2;
   int* tauA = reinterpret_cast<int*>(gbase);
   __nv_bfloat16* A = reinterpret_cast<__nv_bfloat16*>(gbase + ((Mmax * sizeof(int) + 255) & ~size_t(255)));
-  cudaError_t e = launch_k(oz_scale_kernel, dim3(2 * d), dim3(256), 0, s, P, d, tauP, sigP, err);
-  const unsigned eb = (unsigned)std::min<int64_t>((dd + 255) / 256, 152 * 16);
+  cudaError_t e = launch_k(oz_scale_kernel, dim3((unsigned)oz_scale_ctas(d)), dim3(256), 0, s, P, d, tauP, sigP, err);
   if (e == cudaSuccess)
-    e = launch_k(oz_slice_a_kernel, dim3(eb), dim3(256), 0, s, P, d, (const int*)tauP, B, (float2*)nullptr);
+    e = launch_k(oz_slice_kernel, dim3((unsigned)oz_slice_tiles(d)), dim3(256), 0, s, P, d, (const int*)tauP,
+                 (const int*)sigP, B, (__nv_bfloat16*)nullptr, (float2*)nullptr);
   if (e == cudaSuccess)
     e = launch_k(oz_slice_rows_kernel, dim3((unsigned)std::min<int64_t>(M, 152 * 8)), dim3(256), 0, s,
                  (const double2*)S, M, d, tauA, A, err);
@@ -1200,6 +1218,7 @@ int64_t oz_gate_tiles(const Instance& in, int j) { return ((int64_t(1) << j) / k
 bool oz_gate_items(const Instance& in, char* ws, int j, char* rowbuf, OzItem* pit, RowSliceItem* rit, OzItem* git) {
   // P_j's digits in the squaring's layout (the item of squaring step j + 1 reads P_j)
   if (!oz_square_item(in, ws, j + 1, false, pit)) return false;
+  pit->B = nullptr;  // a gate multiplies by E(P)'s rows only
   const int d = (int)in.d;
   const int64_t M = int64_t(1) << j;
   int* tauA = reinterpret_cast<int*>(rowbuf);
@@ -1225,9 +1244,9 @@ bool oz_gate_items(const Instance& in, char* ws, int j, char* rowbuf, OzItem* pi
 int launch_oz_gate_grouped(const OzItem* pits, const RowSliceItem* rits, const OzItem* gits, const GateRound& R,
                            cudaStream_t s) {
   if (R.g_n <= 0) return 0;
-  const unsigned eb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((R.elems + 255) / 256, 152 * 16));
   cudaError_t e = launch_k(oz_scale_grouped_kernel, dim3((unsigned)R.sblocks), dim3(256), 0, s, pits, R.p_n);
-  if (e == cudaSuccess) e = launch_k(oz_slice_grouped_kernel, dim3(eb), dim3(256), 0, s, pits, R.p_n, R.elems);
+  if (e == cudaSuccess)
+    e = launch_k(oz_slice_grouped_kernel, dim3((unsigned)R.elems), dim3(256), 0, s, pits, R.p_n);
   if (e == cudaSuccess)
     e = launch_k(oz_slice_rows_grouped_kernel, dim3((unsigned)std::min<int64_t>(R.rows, 152 * 16)), dim3(256), 0, s,
                  rits, R.r_n, R.rows);
@@ -1394,9 +1413,9 @@ int64_t oz_square_tiles(const Instance& in) { return (2 * in.d / kBM) * (in.d / 
 int launch_square_oz_grouped(const OzItem* items, int nitems, int64_t sblocks, int64_t elems, int64_t tiles,
                              cudaStream_t s) {
   if (nitems <= 0) return 0;
-  const unsigned eb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((elems + 255) / 256, 152 * 16));
   cudaError_t e = launch_k(oz_scale_grouped_kernel, dim3((unsigned)sblocks), dim3(256), 0, s, items, nitems);
-  if (e == cudaSuccess) e = launch_k(oz_slice_grouped_kernel, dim3(eb), dim3(256), 0, s, items, nitems, elems);
+  if (e == cudaSuccess)
+    e = launch_k(oz_slice_grouped_kernel, dim3((unsigned)elems), dim3(256), 0, s, items, nitems);
   if (e == cudaSuccess)
     e = launch_k(oz_square_grouped_kernel, dim3((unsigned)tiles), dim3(kOzThreads), oz_smem(), s, items, nitems);
   return e == cudaSuccess ? 3 : -1;

@@ -135,6 +135,31 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int chunk) {
   return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4));
 }
 
+// The seven balanced base-256 digits (most significant first) of two integers
+// |F| <= 2^55 from the plain bytes of F + B, B = 128 sum_(s<7) 2^(8 s)
+// (0 <= F + B < 2^57): digit s is byte 6 - s of F + B minus 128 (the top one takes
+// bits 48..56). Each becomes a float by the magic-number form 2^23 + d minus 2^23 + 128
+// (exact), whose upper half is its bf16; w[s] packs digit s of F0 (low half) and
+// F1 (high half).
+__device__ __forceinline__ float byte_digit(uint32_t word, uint32_t sel) {
+  return __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u | sel)) - 8388736.0f;
+}
+__device__ __forceinline__ void digit_words(long long F0, long long F1, uint32_t (&w)[7]) {
+  constexpr unsigned long long kBias = 0x80808080808080ull;
+  const unsigned long long u0 = (unsigned long long)F0 + kBias, u1 = (unsigned long long)F1 + kBias;
+  const uint32_t l0 = (uint32_t)u0, h0 = (uint32_t)(u0 >> 32), l1 = (uint32_t)u1, h1 = (uint32_t)(u1 >> 32);
+  const float t0 = __uint_as_float(0x4B000000u | (h0 >> 16)) - 8388736.0f;
+  const float t1 = __uint_as_float(0x4B000000u | (h1 >> 16)) - 8388736.0f;
+  w[0] = __byte_perm(__float_as_uint(t0), __float_as_uint(t1), 0x7632);
+#pragma unroll
+  for (int s = 1; s < 7; ++s) {
+    const int byte = 6 - s;
+    const float f0 = byte_digit(byte >= 4 ? h0 : l0, (uint32_t)(byte & 3));
+    const float f1 = byte_digit(byte >= 4 ? h1 : l1, (uint32_t)(byte & 3));
+    w[s] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+  }
+}
+
 // mbarrier arrive (one thread)
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
