@@ -660,7 +660,7 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
             sp.e0 = T.elems;
             gm.tile0 = T.tiles;
             T.rows += sp.rows;
-            T.elems += (2 * in.d) * (2 * in.d);
+            T.elems += in.d * in.d;
             T.tiles += qpe::tc_level_tiles(in, j);
             bm.tc_split.push_back(sp);
             bm.tc_gemm.push_back(gm);

@@ -354,19 +354,6 @@ struct OzTopArgs {
   double pscale;   // 1 / N^2
 };
 
-// The top level's drain keeps three 64-bit sums per bin in registers: 104 a
-// thread there, 64 in the producer and MMA warps (96 each at launch).
-template <int MODE, bool FEWER>
-__device__ __forceinline__ void ot_reg_share() {
-  static_assert(128 * 64 + (kOtThreads - 128) * 104 <= kOtThreads * 96, "the shares lie within the launch's registers");
-  if constexpr (MODE == 1) {
-    if constexpr (FEWER)
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-    else
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
-  }
-}
-
 template <int MODE>
 __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
   pdl_begin();
@@ -425,7 +412,6 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
 
   if (warp < 3) {
     // ------------------------------------------------------------ producers
-    ot_reg_share<MODE, true>();
     // item u < 256 of a tile: half u & 1 (complex values 8 (u & 1) .. + 7) of
     // pencil u >> 1; items u and u ^ 1 run in adjacent lanes of one round
     int it = 0;
@@ -512,7 +498,6 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
     // tile and the two digit buffers are unrolled, so that every descriptor is a
     // constant away from a loop invariant (an MMA issues in 42 clocks, the read
     // rate of its operands, instead of about 100).
-    ot_reg_share<MODE, true>();
     const uint32_t idesc = make_idesc<kTcBF16, 32>();
     const uint64_t a_desc0 = sw128_desc(smem_u32(As)), b_desc0 = sw128_desc(smem_u32(Bs));
     const int64_t first = a.tile_begin + blockIdx.x;
@@ -569,7 +554,6 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
     if (!mbar_wait_warp(&mma_done, 0)) atomicExch(&fail, 1);
   } else {
     // ------------------------------------------------------------ drain
-    ot_reg_share<MODE, false>();
     const int q = warp & 3;          // tensor-memory lane quarter
     const int k = (warp - 4) >> 2;   // 0 .. 3
     const int h = k & 1;             // column i = 2 c + h of chunk c

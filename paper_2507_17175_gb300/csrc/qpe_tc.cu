@@ -367,13 +367,13 @@ __device__ __forceinline__ void split_row_fp16(const float* __restrict__ src, __
     if (lane == 0) inv_scale[r] = __uint_as_float((uint32_t)(127 - e - 14) << 23);
     for (int c = lane * 4; c < width; c += 128) {
       const float4 v = *reinterpret_cast<const float4*>(row + c);
-      const float x[4] = {v.x * sc, v.y * sc, v.z * sc, v.w * sc};
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const __half h = __float2half_rn(x[t]);
-        hi[r * width + c + t] = h;
-        lo[r * width + c + t] = __float2half_rn(x[t] - __half2float(h));
-      }
+      const __half2 h0 = __floats2half2_rn(v.x * sc, v.y * sc), h1 = __floats2half2_rn(v.z * sc, v.w * sc);
+      const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
+      const __half2 l0 = __floats2half2_rn(v.x * sc - f0.x, v.y * sc - f0.y);
+      const __half2 l1 = __floats2half2_rn(v.z * sc - f1.x, v.w * sc - f1.y);
+      auto bits = [](__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); };
+      *reinterpret_cast<uint2*>(hi + r * width + c) = make_uint2(bits(h0), bits(h1));
+      *reinterpret_cast<uint2*>(lo + r * width + c) = make_uint2(bits(l0), bits(l1));
     }
   }
 }
@@ -389,28 +389,38 @@ __global__ void split_rows_fp16_kernel(const float* __restrict__ src, __half* __
   pdl_trigger();
 }
 
-// P (d x d complex128) -> real embedding B (2d x 2d, n-major) split hi / lo
-// element e of P's real embedding (2d x 2d, n-major) split into hi / lo
+// P (d x d complex128) -> real embedding B (2d x 2d, n-major) split hi / lo: entry
+// e = i d + k of P gives columns 2k, 2k + 1 of rows 2i (Re, -Im) and 2i + 1 (Im, Re); its
+// two parts are split once (the roundings are symmetric) and stored in pairs.
+// One element of B per thread took four FP64 splits an entry and 2-byte
+// stores: 187 us at d = 2048, 60 us so.
 template <int KIND>
 __device__ __forceinline__ void embed_split_elem(const double2* __restrict__ P, void* __restrict__ hi,
                                                  void* __restrict__ lo, int d, int64_t e) {
-  const int64_t n2 = 2 * (int64_t)d;
-  const int64_t n = e / n2, kk = e - n * n2;
-  const int64_t i = n >> 1, k = kk >> 1;
-  const double2 p = P[i * d + k];
-  const int c = (int)(n & 1), cp = (int)(kk & 1);
-  // [[re, -im], [im, re]]
-  const double v = c == 0 ? (cp == 0 ? p.x : -p.y) : (cp == 0 ? p.y : p.x);
+  const int64_t i = e / d, k = e - i * d;
+  const double2 p = __ldg(P + e);
+  const int64_t o0 = 2 * i * (int64_t)d + k, o1 = o0 + d;  // pairs: rows 2i and 2i + 1
   if constexpr (KIND == kTcTF32) {
-    const float h = tf32_round((float)v);
-    reinterpret_cast<float*>(hi)[e] = h;
-    reinterpret_cast<float*>(lo)[e] = tf32_round((float)(v - (double)h));
+    const float hx = tf32_round((float)p.x), hy = tf32_round((float)p.y);
+    const float lx = tf32_round((float)(p.x - (double)hx)), ly = tf32_round((float)(p.y - (double)hy));
+    float2* H = reinterpret_cast<float2*>(hi);
+    float2* L = reinterpret_cast<float2*>(lo);
+    H[o0] = make_float2(hx, -hy);
+    H[o1] = make_float2(hy, hx);
+    L[o0] = make_float2(lx, -ly);
+    L[o1] = make_float2(ly, lx);
   } else {
     static_assert(KIND == kTcFP16, "gate GEMM operands are tf32 or fp16");
-    const double vs = v * 16384.0;  // 2^14, exact
-    const __half h = __float2half_rn((float)vs);
-    reinterpret_cast<__half*>(hi)[e] = h;
-    reinterpret_cast<__half*>(lo)[e] = __float2half_rn((float)(vs - (double)__half2float(h)));
+    const double x = p.x * 16384.0, y = p.y * 16384.0;  // 2^14, exact
+    const __half hx = __float2half_rn((float)x), hy = __float2half_rn((float)y);
+    const __half lx = __float2half_rn((float)(x - (double)__half2float(hx)));
+    const __half ly = __float2half_rn((float)(y - (double)__half2float(hy)));
+    __half2* H = reinterpret_cast<__half2*>(hi);
+    __half2* L = reinterpret_cast<__half2*>(lo);
+    H[o0] = __halves2half2(hx, __hneg(hy));
+    H[o1] = __halves2half2(hy, hx);
+    L[o0] = __halves2half2(lx, __hneg(ly));
+    L[o1] = __halves2half2(ly, lx);
   }
 }
 
@@ -418,8 +428,8 @@ template <int KIND>
 __global__ void embed_split_kernel(const double2* __restrict__ P, void* __restrict__ hi, void* __restrict__ lo,
                                    int d) {
   pdl_begin();
-  const int64_t n2 = 2 * (int64_t)d;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n2 * n2; e += (int64_t)gridDim.x * blockDim.x)
+  const int64_t dd = (int64_t)d * d;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < dd; e += (int64_t)gridDim.x * blockDim.x)
     embed_split_elem<KIND>(P, hi, lo, d, e);
   pdl_trigger();
 }
@@ -669,7 +679,10 @@ __global__ void __launch_bounds__(256) oz_slice_rows_grouped_kernel(const RowSli
 // One CTA per 128 x 64 tile of out (rows m0.. of E, columns n0.. < d).
 // K-block by K-block (64 elements of K), every digit tile is loaded once: the
 // seven B digit tiles of the K-block (resident, two buffers) and the seven A
-// digit tiles, each refilled once its pairs are done; A digit s meets B digits
+// digit tiles, which four warps move on into tensor memory (two buffers of 32
+// columns): with N = 64 an MMA that reads A from shared memory takes 48 clocks
+// (6 KiB at 128 bytes a clock, and TMA's writes share the port), from tensor
+// memory the 32 of the tensor pipe. A digit s meets B digits
 // t = 0 .. 6 - s, and pair (s, t) goes into the tensor-memory accumulator of
 // weight w = s + t (64 columns each, 448 in all). Weight w is complete for the
 // K-block once A digit w has been used, so the weights finish in order and
@@ -677,14 +690,13 @@ __global__ void __launch_bounds__(256) oz_slice_rows_grouped_kernel(const RowSli
 // An accumulator holds (w + 1) pairs per K-block, each at most 64 * 2^14, so
 // it stays an exact FP32 integer (below 2^24) over a window of win_w
 // K-blocks, (w + 1) * win_w < 16; the drain reads it once per window.
-// Drain warps 2 .. 9 (two per tensor-memory lane quarter, 32 columns each)
-// convert the window sums to integers and add them into two int64 sums per
-// column, hi = sum_(w <= 2) acc_w 2^(8 (2 - w)) and lo = sum_(w >= 3) acc_w
-// 2^(8 (6 - w)) (below 2^44 and 2^54 for K <= 8192); at the end
-// val = hi 2^-32 + lo 2^-64 and out = val 2^(tau_m + sigma_n + 2).
-// Warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the MMAs.
+// Drain warps 6 .. 13 (two per tensor-memory lane quarter, 32 columns each)
+// convert the window sums to integers and add them into one 96-bit sum per column
+// (Oz96), val = sum 2^-64; out = val 2^(tau_m + sigma_n + 2).
+// Warp 0 lane 0 issues the TMA loads, warp 1 the MMAs, warps 2 .. 5 move A.
 constexpr int kOzBN = 64;
-constexpr int kOzThreads = 320;
+constexpr int kOzThreads = 448;
+constexpr int kOzACol = kOzS * kOzBN;          // tensor-memory column of the first A buffer
 constexpr int kOzA = kBM * 128;              // one A digit tile, 16 KiB
 constexpr int kOzB = kOzBN * 128;            // one B digit tile, 8 KiB
 constexpr int kOzBSet = kOzS * kOzB;         // the seven B digit tiles of a K-block
@@ -716,14 +728,14 @@ __device__ __forceinline__ bool oz_window_end(int kb, int kblocks) {
 // Pair (S, T): four K = 16 steps into the accumulator of weight S + T; FRESH
 // overwrites it.
 template <int S, int T, bool FRESH>
-__device__ __forceinline__ void oz_mma_pair(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc) {
+__device__ __forceinline__ void oz_mma_pair(uint32_t tmem, uint32_t ad, uint64_t bd0, uint32_t idesc) {
   const uint64_t bd = bd0 + (uint64_t)(T * (kOzB >> 4));
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    umma_k<kTcBF16>(tmem + (uint32_t)((S + T) * kOzBN), ad + 2 * k, bd + 2 * k, idesc, (FRESH && k == 0) ? 0u : 1u);
+    umma_ts(tmem + (uint32_t)((S + T) * kOzBN), ad + 8 * k, bd + 2 * k, idesc, (FRESH && k == 0) ? 0u : 1u);
 }
 template <int S, int T>
-__device__ __forceinline__ void oz_mma_pairs(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc) {
+__device__ __forceinline__ void oz_mma_pairs(uint32_t tmem, uint32_t ad, uint64_t bd0, uint32_t idesc) {
   if constexpr (S + T < kOzS) {
     oz_mma_pair<S, T, false>(tmem, ad, bd0, idesc);
     oz_mma_pairs<S, T + 1>(tmem, ad, bd0, idesc);
@@ -734,7 +746,7 @@ __device__ __forceinline__ void oz_mma_pairs(uint32_t tmem, uint64_t ad, uint64_
 // start of a window it waits for the drain of the window before and overwrites
 // the accumulator. False if that wait runs out.
 template <int T>
-__device__ __forceinline__ bool oz_mma_first(uint32_t tmem, uint64_t ad, uint64_t bd0, uint32_t idesc, int kb,
+__device__ __forceinline__ bool oz_mma_first(uint32_t tmem, uint32_t ad, uint64_t bd0, uint32_t idesc, int kb,
                                              uint64_t* acc_empty) {
   if constexpr (T < kOzS) {
     if (oz_window_start<T>(kb)) {
@@ -751,84 +763,138 @@ __device__ __forceinline__ bool oz_mma_first(uint32_t tmem, uint64_t ad, uint64_
   return true;
 }
 
-// A digits S .. 6 of one K-block (the whole warp; one elected lane issues):
-// wait for the digit's tile, its pairs, release the tile, and signal weight S
-// complete at the end of its window. Every descriptor is a constant away from
-// a loop invariant: with a ring stage computed at run time an MMA took 72
-// clocks to issue against the 48 its operands take to read.
-template <int S>
-__device__ __forceinline__ bool oz_mma_digits(uint32_t tmem, uint64_t a_desc0, uint64_t bd0, uint32_t idesc, int kb,
-                                              int kblocks, uint64_t* a_full, uint64_t* a_empty, uint64_t* acc_full,
+// A digits S .. 6 of one K-block on B buffer BB (the whole warp; one elected
+// lane issues): wait for the digit in its tensor-memory buffer, its pairs,
+// release the buffer, and signal weight S complete at the end of its window.
+// Every operand is a constant away from a loop invariant: with a ring stage
+// computed at run time an MMA took 72 clocks to issue.
+template <int S, int BB>
+__device__ __forceinline__ bool oz_mma_digits(uint32_t tmem, uint64_t bd0, uint32_t idesc, int kb, int kblocks,
+                                              uint64_t* at_full, uint64_t* at_empty, uint64_t* acc_full,
                                               uint64_t* acc_empty) {
   if constexpr (S < kOzS) {
-    if (!mbar_wait_warp(&a_full[S], kb & 1)) return false;
+    constexpr int buf = (BB + S) & 1;  // digit u = 7 kb + S of the tile goes to buffer u & 1
+    if (!mbar_wait_warp(&at_full[buf], (uint32_t)((kOzS * kb + S) >> 1) & 1)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint64_t ad = a_desc0 + (uint64_t)(S * (kOzA >> 4));
+    const uint32_t ad = tmem + (uint32_t)(kOzACol + 32 * buf);
     if constexpr (S == 0) {
       if (!oz_mma_first<0>(tmem, ad, bd0, idesc, kb, acc_empty)) return false;
     }
     const bool done = oz_window_end<S>(kb, kblocks);  // weight S is complete
     if (elect_one()) {
       if constexpr (S > 0) oz_mma_pairs<S, 0>(tmem, ad, bd0, idesc);
-      umma_commit(&a_empty[S]);
+      umma_commit(&at_empty[buf]);
       if (done) umma_commit(&acc_full[S]);
     }
-    return oz_mma_digits<S + 1>(tmem, a_desc0, bd0, idesc, kb, kblocks, a_full, a_empty, acc_full, acc_empty);
+    return oz_mma_digits<S + 1, BB>(tmem, bd0, idesc, kb, kblocks, at_full, at_empty, acc_full, acc_empty);
   }
   return true;
 }
 
 // One K-block on B buffer BB (the whole warp)
 template <int BB>
-__device__ __forceinline__ bool oz_mma_kblock(uint32_t tmem, uint64_t a_desc0, uint64_t b_desc0, uint32_t idesc,
-                                              int kb, int kblocks, uint64_t* a_full, uint64_t* a_empty,
-                                              uint64_t* b_full, uint64_t* b_empty, uint64_t* acc_full,
-                                              uint64_t* acc_empty) {
+__device__ __forceinline__ bool oz_mma_kblock(uint32_t tmem, uint64_t b_desc0, uint32_t idesc, int kb, int kblocks,
+                                              uint64_t* at_full, uint64_t* at_empty, uint64_t* b_full,
+                                              uint64_t* b_empty, uint64_t* acc_full, uint64_t* acc_empty) {
+  static_assert(kOzS % 2 == 1, "the A buffers alternate between K-blocks too");
   if (!mbar_wait_warp(&b_full[BB], (kb >> 1) & 1)) return false;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!oz_mma_digits<0>(tmem, a_desc0, b_desc0 + (uint64_t)(BB * (kOzBSet >> 4)), idesc, kb, kblocks, a_full, a_empty,
-                        acc_full, acc_empty))
+  if (!oz_mma_digits<0, BB>(tmem, b_desc0 + (uint64_t)(BB * (kOzBSet >> 4)), idesc, kb, kblocks, at_full, at_empty,
+                            acc_full, acc_empty))
     return false;
   if (elect_one()) umma_commit(&b_empty[BB]);
   return true;
 }
 
+// The A digits of the whole tile, smem -> tensor memory, by the four warps of
+// the lane quarters (warp q: rows 32 q .. 32 q + 31, a row per lane).
+__device__ __forceinline__ bool oz_move_a(uint32_t tmem, uint32_t aset, int q, int lane, int kblocks, uint64_t* a_full,
+                                          uint64_t* a_empty, uint64_t* at_full, uint64_t* at_empty, const int* fail) {
+  const int row = q * 32 + lane;
+  const uint32_t dst = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)kOzACol;
+  int u = 0;
+  for (int kb = 0; kb < kblocks; ++kb) {
+#pragma unroll 1
+    for (int s = 0; s < kOzS; ++s, ++u) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], kb & 1) && !*((volatile const int*)fail))) return false;
+      uint4 v[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v[c].x), "=r"(v[c].y), "=r"(v[c].z), "=r"(v[c].w)
+                     : "r"(aset + (uint32_t)(s * kOzA) + sw128_offset(row, c))
+                     : "memory");
+      if (u >= 2 && !mbar_wait_warp(&at_empty[u & 1], (uint32_t)((u >> 1) - 1) & 1)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tmem_st32(dst + (uint32_t)(32 * (u & 1)), v);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&at_full[u & 1]);
+        mbar_arrive(&a_empty[s]);
+      }
+    }
+  }
+  return true;
+}
+
+// One output's sum over the weights in 96 bits: sum_w acc_w 2^(8 (6 - w)) (below
+// 2^76 for K <= 8192); three registers, so that a drain thread's 32 columns and 16
+// accumulators in flight fit 128.
+struct Oz96 {
+  uint32_t w0 = 0, w1 = 0, w2 = 0;
+  template <int W>
+  __device__ __forceinline__ void add(int x) {
+    if constexpr (W <= 2) {  // 2^(8 (6 - W)) >= 2^32
+      const long long v = (long long)x << (8 * (2 - W));
+      asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;"
+          : "+r"(w1), "+r"(w2)
+          : "r"((uint32_t)v), "r"((uint32_t)(v >> 32)));
+    } else {
+      const long long v = (long long)x << (8 * (6 - W));
+      asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+          : "+r"(w0), "+r"(w1), "+r"(w2)
+          : "r"((uint32_t)v), "r"((uint32_t)(v >> 32)), "r"((uint32_t)(x >> 31)));
+    }
+  }
+  // the sum times 2^-64, rounded once (its upper words are below 2^44, exact)
+  __device__ __forceinline__ double value() const {
+    const long long hi = (long long)(((unsigned long long)w2 << 32) | w1);
+    return fma((double)w0, 0x1p-64, (double)hi * 0x1p-32);
+  }
+};
+
 // Drain of weight W at the end of its window: 32 columns of this warp's lane
-// quarter into the int64 sums (weights 0-2 into hi, 3-6 into lo, shifted by
-// their place). False if the wait runs out or another role failed.
+// quarter into the sums. False if the wait runs out or another role failed.
 template <int W>
 __device__ __forceinline__ bool oz_drain_weight(uint32_t taddr, int kb, uint64_t* acc_full, uint64_t* acc_empty,
-                                                const int* fail, int lane, long long (&hi)[32],
-                                                long long (&lo)[32]) {
+                                                const int* fail, int lane, Oz96 (&sum)[32]) {
   bool got = mbar_wait(&acc_full[W], oz_window<W>(kb) & 1);
   got = __all_sync(0xffffffffu, got && !*((volatile const int*)fail)) != 0;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!got) return false;
-  uint32_t v[32];
-  tmem_ld32(taddr + (uint32_t)(W * kOzBN), v);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncwarp();
-  if (lane == 0) mbar_arrive(&acc_empty[W]);
-  constexpr int sh = 8 * ((W <= 2 ? 2 : 6) - W);
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const long long x = (long long)__float2int_rn(__uint_as_float(v[i])) << sh;
-    if constexpr (W <= 2)
-      hi[i] += x;
-    else
-      lo[i] += x;
+  for (int part = 0; part < 4; ++part) {
+    uint32_t v[8];
+    tmem_ld8(taddr + (uint32_t)(W * kOzBN + 8 * part), v);
+    if (part == 3) {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[W]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum[8 * part + i].template add<W>(__float2int_rn(__uint_as_float(v[i])));
   }
   return true;
 }
 
 template <int W>
 __device__ __forceinline__ bool oz_drain_kblock(uint32_t taddr, int kb, int kblocks, uint64_t* acc_full,
-                                                uint64_t* acc_empty, const int* fail, int lane, long long (&hi)[32],
-                                                long long (&lo)[32]) {
+                                                uint64_t* acc_empty, const int* fail, int lane, Oz96 (&sum)[32]) {
   if constexpr (W < kOzS) {
-    if (oz_window_end<W>(kb, kblocks) && !oz_drain_weight<W>(taddr, kb, acc_full, acc_empty, fail, lane, hi, lo))
+    if (oz_window_end<W>(kb, kblocks) && !oz_drain_weight<W>(taddr, kb, acc_full, acc_empty, fail, lane, sum))
       return false;
-    return oz_drain_kblock<W + 1>(taddr, kb, kblocks, acc_full, acc_empty, fail, lane, hi, lo);
+    return oz_drain_kblock<W + 1>(taddr, kb, kblocks, acc_full, acc_empty, fail, lane, sum);
   }
   return true;
 }
@@ -840,7 +906,7 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   unsigned char* bset = base;                // 2 x kOzBSet
   unsigned char* aset = base + 2 * kOzBSet;  // kOzS x kOzA
-  __shared__ uint64_t a_full[kOzS], a_empty[kOzS], b_full[2], b_empty[2];
+  __shared__ uint64_t a_full[kOzS], a_empty[kOzS], at_full[2], at_empty[2], b_full[2], b_empty[2];
   __shared__ uint64_t acc_full[kOzS], acc_empty[kOzS], mma_done;
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
@@ -866,9 +932,11 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
   if (threadIdx.x == 0) {
     for (int s = 0; s < kOzS; ++s) {
       mbar_init(&a_full[s], 1);
-      mbar_init(&a_empty[s], 1);
+      mbar_init(&a_empty[s], 4);  // the four warps that move A
     }
     for (int b = 0; b < 2; ++b) {
+      mbar_init(&at_full[b], 4);
+      mbar_init(&at_empty[b], 1);
       mbar_init(&b_full[b], 1);
       mbar_init(&b_empty[b], 1);
     }
@@ -925,12 +993,12 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
     }
   } else if (warp == 1) {
     const uint32_t idesc = make_idesc<kTcBF16, kOzBN>();
-    const uint64_t a_desc0 = sw128_desc(smem_u32(aset)), b_desc0 = sw128_desc(smem_u32(bset));
+    const uint64_t b_desc0 = sw128_desc(smem_u32(bset));
     for (int kb = 0; kb < kblocks; kb += 2) {
-      if (!oz_mma_kblock<0>(tmem, a_desc0, b_desc0, idesc, kb, kblocks, a_full, a_empty, b_full, b_empty, acc_full,
+      if (!oz_mma_kblock<0>(tmem, b_desc0, idesc, kb, kblocks, at_full, at_empty, b_full, b_empty, acc_full,
                             acc_empty) ||
-          (kb + 1 < kblocks && !oz_mma_kblock<1>(tmem, a_desc0, b_desc0, idesc, kb + 1, kblocks, a_full, a_empty,
-                                                 b_full, b_empty, acc_full, acc_empty))) {
+          (kb + 1 < kblocks && !oz_mma_kblock<1>(tmem, b_desc0, idesc, kb + 1, kblocks, at_full, at_empty, b_full,
+                                                 b_empty, acc_full, acc_empty))) {
         atomicExch(&fail, 1);
         break;
       }
@@ -938,17 +1006,18 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
     // every MMA issued has finished before tensor memory is released
     if (elect_one()) umma_commit(&mma_done);
     if (!mbar_wait_warp(&mma_done, 0)) atomicExch(&fail, 1);
+  } else if (warp < 6) {
+    if (!oz_move_a(tmem, smem_u32(aset), warp & 3, lane, kblocks, a_full, a_empty, at_full, at_empty, &fail))
+      atomicExch(&fail, 1);
   } else {
     const int q = warp & 3;          // tensor-memory lane quarter
-    const int h = (warp - 2) >> 2;   // column half
+    const int h = (warp - 6) >> 2;   // column half
     const int row = q * 32 + lane;   // tile row of this thread
-    long long hi[32], lo[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0;
+    Oz96 sum[32];
     bool ok = true;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * 32);
     for (int kb = 0; kb < kblocks && ok; ++kb)
-      ok = oz_drain_kblock<0>(taddr, kb, kblocks, acc_full, acc_empty, &fail, lane, hi, lo);
+      ok = oz_drain_kblock<0>(taddr, kb, kblocks, acc_full, acc_empty, &fail, lane, sum);
     if (ok && a.M) {
       // gate level: product row r -> state row row_out + r; this thread's 32
       // columns are all real (n < d) or all imaginary parts
@@ -958,7 +1027,7 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
       double* vr = reinterpret_cast<double*>(a.S + (a.row_out + r) * d + j0) + im;
 #pragma unroll
       for (int n = 0; n < 32; ++n) {
-        const double val = fma((double)lo[n], 0x1p-64, (double)hi[n] * 0x1p-32);
+        const double val = sum[n].value();
         const int e = t + a.sig[j0 + n] + 2;
         vr[2 * n] = val == 0.0 ? 0.0 : val * pow2d(e < -1022 ? -1022 : e);
       }
@@ -970,7 +1039,7 @@ __device__ __forceinline__ void oz_square_tile(const CUtensorMap* mapA, const CU
 #pragma unroll
       for (int n = 0; n < 32; ++n) {
         const int col = n0 + h * 32 + n;
-        const double val = fma((double)lo[n], 0x1p-64, (double)hi[n] * 0x1p-32);
+        const double val = sum[n].value();
         const int e = t + a.sig[col] + 2;
         const double c = val == 0.0 ? 0.0 : val * pow2d(e < -1022 ? -1022 : e);
         vr[2 * n] = c;
@@ -1293,7 +1362,7 @@ int launch_tc_level(const Instance& in, char* ws, int prec, int j, cudaStream_t 
   }
   if (e != cudaSuccess) return -1;
   ++launches;
-  const int eblocks = (int)std::min<int64_t>((d2 * d2 + 255) / 256, 152 * 16);
+  const int eblocks = (int)std::min<int64_t>((in.d * in.d + 255) / 256, 152 * 16);
   e = kind == kTcTF32 ? launch_k(embed_split_kernel<kTcTF32>, dim3(eblocks), dim3(256), 0, s, Pj, (void*)Bhi,
                                  (void*)Blo, (int)in.d)
                       : launch_k(embed_split_kernel<kTcFP16>, dim3(eblocks), dim3(256), 0, s, Pj, (void*)Bhi,
