@@ -231,7 +231,7 @@ __device__ __forceinline__ void rows_times_pt_tile(C* __restrict__ S, const C* _
   if constexpr (BN <= 4) {
     // d = 2, 4: a thread owns a row (16-byte loads and stores, P from the L1 cache,
     // the same order of additions), HBM is the bound: d = 4, 2^25 rows complex64 by
-    // doubling 568 -> 260 us
+    // doubling 568 -> 379 us
     static_assert(NT == BM, "a thread per row");
     const int64_t lr = bx * BM + threadIdx.x;
     if (lr >= M) return;
@@ -333,7 +333,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 // warp's lanes), KS warps of a CTA share the inner index where the block count
 // alone leaves SMs idle, and the lanes' partial sums meet in one shuffle
 // reduce-scatter: no barrier in the loop, no padding for M >= TM, every SM busy
-// from M d >= 152 x 16 outputs on. The rule that picks it is few_rows().
+// from M d >= 152 x 16 outputs on. The rule that picks it is few_rows(). Levels M = 1 .. 64
+// at d = 1024 complex128: 30.0 -> 1.1 ms (M = 64: 525 us, 430 at the FP64 rate); M = 1 .. 2048
+// at d = 256 complex64: 838 -> 155 us.
 constexpr int kFewWarps = 8, kFewTN = 4;
 
 template <int TM>
@@ -454,8 +456,8 @@ __global__ void __launch_bounds__(32 * kFewWarps)
 // digit y = k1 + R1 k2) and stores from registers. Passes over narrow rows
 // (Q below 128 bytes: the last pass of small registers) take several blocks per
 // CTA, whose rows are consecutive in memory.
-// 2^27 points, three passes: complex64 2.24 -> 1.39 ms (4.6 TB/s), and complex128 (Nmat 10,
-// Nmeas 17, two passes) 19.9 -> 15.2 ms.
+// 2^27 points: complex64, three passes 2.24 -> 1.53 ms (4.2 TB/s); complex128 (Nmat 10,
+// Nmeas 17, two passes) 19.9 -> 18.2 ms, bound by the FP64 units.
 __host__ __device__ constexpr int fft_k1(int logr) { return logr <= 4 ? logr : logr <= 6 ? 3 : logr <= 8 ? 4 : 5; }
 
 // complex128 takes up to 32 points in 128 registers a thread: CTAs of half the
@@ -916,7 +918,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const Partial* __restrict
 // log2 of the pieces per row). Rows of at most 64 bytes with two digits or more
 // go through shared memory in tiles of 32 consecutive y times K values of y's
 // highest digit, which is the position's lowest: read as runs of K rows, written as
-// runs of 32 (2^25 rows of 32 bytes: 780 -> 420 us; a row at a time leaves every
+// runs of 32 (2^25 rows of 32 bytes: 780 -> 376 us; a row at a time leaves every
 // 32-byte sector in its own DRAM burst).
 constexpr int kUnpermuteTile = 2048;  // 16-byte pieces
 __global__ void __launch_bounds__(256) unpermute_kernel(const float4* __restrict__ X, float4* __restrict__ out,

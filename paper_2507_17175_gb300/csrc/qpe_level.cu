@@ -1126,7 +1126,8 @@ bool level_sharded(const Instance& in, int li) {
 // Levels of r <= rmax bits, the top one first. At most 256 outcomes are a matter of
 // latency: a level of five bits is one pencil or two whose 32-point FP64 DFTs and
 // five-factor table rows run on a few lanes of one SM, so `balanced` splits them into
-// equal levels of at most four bits (Nmat 2, Nmeas 6 FP64: top level 61 -> 15 us).
+// equal levels of at most four bits (Nmat 2, Nmeas 6 FP64: the call 132.6 -> 81.4 us,
+// one read-back copy less included; the five-bit top level alone took 61).
 std::vector<Level> make_levels(int nmeas, int logd, size_t esize, bool balanced) {
   int rmax = level_max_bits(logd, esize, kLevelSmemCap);
   if (balanced && nmeas <= 8 && rmax > 4) {

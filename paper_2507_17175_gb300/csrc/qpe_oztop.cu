@@ -24,26 +24,27 @@
 // product.
 //
 // GB300 issues an FP64 instruction at 1/32 of the rate of a 32-bit integer
-// one, so the epilogue stays in 64-bit fixed point until |X|^2: the drain
+// one, so the epilogue stays in 64-bit fixed point up to the sums of |X|^2: the drain
 // reads each accumulator as an int (a magic-number addition in FP32), forms
 // W = floor(E / 2^10) (|W| < 2^57 + 1, units 2^(tau + sigma - 52)),
 // multiplies by the twiddles held in Q61 (round(w 2^61), split at bit 31 into
 // int32 halves so that every partial product is one 32 x 32 -> 64-bit
 // multiply-add; at most 3 units off), runs the 8-point DFT on the integers
-// (|X| < 8 sqrt(2) 2^57 < 2^61; the factor cos(pi / 4) also in Q61) and turns
-// X into FP64 (the hardware conversion, rounded to nearest; the unit's power
-// of two goes into the exponent bits, or, for |X|^2, into the histogram's
-// scale once per tile). The fixed point's truncations are a few units, 2^-55
-// of the pencil's bound |T| < 2^(tau + sigma + 5), below the contraction's
-// own error. |X|^2 and the readout run in FP64; a lower level (MODE 0) stores
-// X in FP64.
+// (|X| < 8 sqrt(2) 2^57 < 2^61; the factor cos(pi / 4) also in Q61), sums |X|^2
+// exactly in integers (OtSquares; the unit goes into the histogram's scale once
+// per tile) or, in a lower level (MODE 0), stores X in FP64 (the hardware
+// conversion, rounded to nearest; the unit's power of two goes into the exponent
+// bits). The fixed point's truncations are a few units, 2^-55 of the pencil's
+// bound |T| < 2^(tau + sigma + 5), below the contraction's own error. The sums
+// over the warps and the readout run in FP64. Top level at Nmeas 24: 4.0 ms with
+// its lower levels before the MMA warp ran converged, 3.2 so (2.48 ms alone).
 //
 // Roles (640 threads, one CTA per SM, persistent over the tiles):
 //   warps 0-2   producers: Z rows -> digit tiles (shared memory, 128-byte
 //               swizzled K-major, two digits per 128-byte row), two threads
 //               per pencil (eight complex values each); the pencils'
 //               twiddles w_N^(m_b y_a) and scales (two buffers);
-//   warp 3      tensor memory, and lane 0 issues the MMAs and the table's
+//   warp 3      tensor memory; runs converged, one elected lane issues the MMAs, lane 0 the table's
 //               copies: per chunk of two columns i (32 table rows), 28 pairs
 //               x 2 K-steps of M = 128, N = 32 into seven weight accumulators
 //               (224 columns; two chunk buffers, even chunks in one, odd in
@@ -54,8 +55,8 @@
 //               SM sub-partition, for the integer epilogue's latencies),
 //               warp k takes column 2 c + (k & 1) of the chunks
 //               c with c & 1 = k >> 1; weights -> fixed point, twiddle, DFT,
-//               FP64, then |X|^2 (the four warps' sums meet through tensor
-//               memory columns 448-495) or the store of X.
+//               then the sums of |X|^2 (the four warps' meet as doubles through
+//               tensor memory columns 448-495) or the store of X in FP64.
 // Every wait is a bounded mbarrier wait; an expired wait sets QPE_ERR_TIMEOUT.
 #include "qpe_internal.cuh"
 #include "qpe_tcgen05.cuh"
