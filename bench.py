@@ -414,7 +414,7 @@ def bench_ours(args, rank, world, local_rank):
         roofline = {"bound": "hbm", "achieved": round(ach, 1), "peak": round(pk["hbm_gbs"], 1),
                     "unit": "GB/s", "frac": round(ach / pk["hbm_gbs"], 4),
                     "traffic": recorded_traffic("level_oz_top_c5_fp64"),
-                    "kernel": "level_oz_kernel<1> (tcgen05 digit products + fixed-point twiddle / DFT, FP64 |X|^2)",
+                    "kernel": "level_oz_kernel<1> (tcgen05 digit products + fixed-point twiddle / DFT, integer |X|^2)",
                     "kernel_ms": round(t_k, 3), "algorithmic_bytes_per_launch": alg_bytes,
                     "algorithmic_bytes": f"2 x state bytes = 2 x 2^{n} x {d} x 16 B (the C5 roofline's 2 S_B: "
                                          "final state written once and read once)",
