@@ -284,6 +284,15 @@ def _ptr(x):
     raise TypeError(f"unsupported buffer type {type(x)}")
 
 
+def _order_after_current(stream, device):
+    """What qpe_bind enqueues on ``stream`` waits for the current stream: torch
+    hands out workspace memory whose last user there may still be running."""
+    import torch
+    current = torch.cuda.current_stream(device)
+    if stream.cuda_stream != current.cuda_stream:
+        stream.wait_stream(current)
+
+
 class Plan:
     """One QPE problem bound to a torch-allocated workspace and stream."""
 
@@ -303,6 +312,7 @@ class Plan:
         if workspace is None:
             workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = workspace
+        _order_after_current(stream, self.device)
         self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
 
     # -------------------------------------------------------------- helpers
@@ -440,6 +450,7 @@ class ShardedPlan(Plan):
         if workspace is None:
             workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = workspace
+        _order_after_current(stream, self.device)
         self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
 
     def probs(self, out=None, instance: int = 0, want_hist: bool = True):
@@ -524,6 +535,7 @@ class BatchedPlan(Plan):
             workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = workspace
         self._keep_inputs = {}
+        _order_after_current(stream, self.device)
         self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
 
     def load(self, instance: int, U, psi):
