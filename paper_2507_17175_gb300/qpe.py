@@ -284,12 +284,23 @@ def _ptr(x):
     raise TypeError(f"unsupported buffer type {type(x)}")
 
 
-def _order_after_current(stream, device):
-    """What qpe_bind enqueues on ``stream`` waits for the current stream: torch
-    hands out workspace memory whose last user there may still be running."""
+def _other_current(stream, device):
+    """The current stream where it is another one than ``stream``, else None.
+    None too while it is being captured: an event of a capture cannot order work
+    outside of it, and waiting for one would draw ``stream`` into the capture."""
     import torch
     current = torch.cuda.current_stream(device)
-    if stream.cuda_stream != current.cuda_stream:
+    if stream.cuda_stream == current.cuda_stream or torch.cuda.is_current_stream_capturing():
+        return None
+    return current
+
+
+def _order_after_current(stream, device):
+    """What is enqueued on ``stream`` from here on waits for the current stream:
+    a caller's tensors are written there, and torch hands out memory whose last
+    user there may still be running."""
+    current = _other_current(stream, device)
+    if current is not None:
         stream.wait_stream(current)
 
 
@@ -343,6 +354,8 @@ class Plan:
         pp, dp = _ptr(psi)
         if du != dp:
             raise ValueError("U and psi must both be host or both be device buffers")
+        if du:
+            _order_after_current(self.stream, self.device)
         self._keep = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, self.nmat, self.nmeas, du), "qpe_load")
 
@@ -387,6 +400,8 @@ class Plan:
         if isinstance(S, np.ndarray):
             S = np.ascontiguousarray(S, dtype=self.state_dtype)
         ptr, dev = _ptr(S)
+        if dev:
+            _order_after_current(self.stream, self.device)
         self._keep_state = S
         self._check(_lib.qpe_load_state(self._h, instance, ptr, dev), "qpe_load_state")
 
@@ -545,6 +560,8 @@ class BatchedPlan(Plan):
             psi = np.ascontiguousarray(psi, dtype=np.complex128)
         pu, du = _ptr(U)
         pp, dp = _ptr(psi)
+        if du:
+            _order_after_current(self.stream, self.device)
         self._keep_inputs[instance] = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, nmat, nmeas, du), "qpe_load")
 
