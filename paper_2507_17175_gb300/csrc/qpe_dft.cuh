@@ -7,9 +7,11 @@
 namespace qpe {
 
 // v exp(-2 pi i K / 32) for a compile-time K in 0 .. 15 after unrolling: nothing
-// for 0, an exchange for 8, two additions and two multiplications for 4 and 12
+// for 0, an exchange for 8, else a product and an FMA for each part. (x +- y) cos(pi / 4)
+// for 4 and 12 takes as many operations and rounds the sum before the product: 2 to 4%
+// more rms error in a complex64 DFT of 8 to 32 points.
 template <typename C>
-__device__ __forceinline__ C rot32(C v, int K) {
+__host__ __device__ __forceinline__ C rot32(C v, int K) {
   using R_t = typename real_of<C>::type;
   constexpr double cs[9] = {1.0,
                             0.98078528040323044913,  // cos(pi k / 16)
@@ -22,17 +24,14 @@ __device__ __forceinline__ C rot32(C v, int K) {
                             0.0};
   if (K == 0) return v;
   if (K == 8) return mk(v.y, -v.x);
-  const R_t c4 = (R_t)cs[4];
-  if (K == 4) return mk((v.x + v.y) * c4, (v.y - v.x) * c4);
-  if (K == 12) return mk((v.y - v.x) * c4, -((v.x + v.y) * c4));
   const R_t c = (R_t)(K < 8 ? cs[K & 7] : -cs[(16 - K) & 7]), s = (R_t)(K < 8 ? cs[8 - (K & 7)] : cs[K & 7]);
   // s = sin(pi K / 16): cos(pi (8 - K) / 16) for K < 8, cos(pi (K - 8) / 16) above
-  return mk(v.x * c + v.y * s, v.y * c - v.x * s);
+  return mk(fma(v.x, c, v.y * s), fma(v.y, c, -(v.x * s)));
 }
 
 // X[k] = sum_n x[n] exp(-2 pi i n k / 2^K) of x[0 .. 2^K), natural order in and out
 template <typename C, int K, int N>
-__device__ __forceinline__ void dft_k(C (&x)[N]) {
+__host__ __device__ __forceinline__ void dft_k(C (&x)[N]) {
   constexpr int R = 1 << K;
 #pragma unroll
   for (int s = 0; s < K; ++s) {
