@@ -698,8 +698,20 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
       }
       int maxp = 0;
       for (int i : pl) maxp = std::max(maxp, p->inst[i].fft.passes);
-      for (int pass = 0; pass < maxp; ++pass) {
+      // A pass's short transforms and the others: two kernels, two rounds. Next to a long
+      // transform every one goes with it (a launch more costs 5 us), and next to passes of
+      // 9 bits in complex128 that fill a tile: those take 55 us there, 59 so when grouped.
+      for (int round = 0; round < 2 * maxp; ++round) {
+        const int pass = round / 2;
+        const bool tiles = std::any_of(pl.begin(), pl.end(), [&](int i) {
+          int64_t nb = 0;
+          size_t sm = 0;
+          const qpe::FftPlan& f = p->inst[i].fft;
+          return f.passes > pass && ((!c64 && f.p[pass].logr == 9 && f.p[pass].Q >= 8) ||
+                                     !qpe::fft_pass_args(p->inst[i], pass, &nb, &sm, sizeof(C)).small);
+        });
         qpe::FftRound R{};
+        R.small = round % 2;
         R.item_off = (int)(bm.fft_items.size() / sizeof(qpe::FftItem<C>));
         int64_t blocks = 0;
         size_t smem = 0;
@@ -709,7 +721,8 @@ void build_batch_meta(qpe_plan_t p, char* ws, int nsm) {
           qpe::FftItem<C> it{};
           int64_t nb = 0;
           size_t sm = 0;
-          it.a = qpe::fft_pass_args(in, pass, &nb, &sm, sizeof(C));
+          it.a = qpe::fft_pass_args(in, pass, &nb, &sm, sizeof(C), tiles);
+          if (it.a.small != R.small) continue;
           it.X = reinterpret_cast<C*>(ws + in.off_state);
           it.lo = reinterpret_cast<const C*>(ws + (c64 ? in.off_tw_lo32 : in.off_tw_lo64));
           it.hi = reinterpret_cast<const C*>(ws + (c64 ? in.off_tw_hi32 : in.off_tw_hi64));
@@ -972,7 +985,7 @@ qpe_status enqueue_batched(qpe_plan_t p, int64_t* launches) {
       if (!mark(2)) return false;
       for (const qpe::FftRound& R : bm.fft_rounds)
         if (!chk(qpe::launch_fft_grouped<C>(reinterpret_cast<const qpe::FftItem<C>*>(ws + bm.off_fft) + R.item_off,
-                                            R.nitems, R.blocks, R.smem, p->stream)))
+                                            R.nitems, R.blocks, R.smem, R.small, p->stream)))
           return false;
       if (!mark(3)) return false;
       if (!chk(qpe::launch_reduce_grouped<C>(reinterpret_cast<const qpe::RedItem<C>*>(ws + bm.off_red), bm.nred,

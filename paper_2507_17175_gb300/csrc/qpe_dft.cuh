@@ -66,11 +66,17 @@ __host__ __device__ __forceinline__ void dft_k(C (&x)[N]) {
   }
 }
 
+// A butterfly's difference times its twiddle, in a table-driven transform. complex64:
+// the roundings are written out, so that they do not depend on how the surrounding code is
+// compiled.
+__device__ __forceinline__ float2 twiddled(float2 d, float2 w) {
+  return mk(__fmaf_rn(d.x, w.x, -__fmul_rn(d.y, w.y)), __fmaf_rn(d.y, w.x, __fmul_rn(d.x, w.y)));
+}
+__device__ __forceinline__ double2 twiddled(double2 d, double2 w) { return cmul(d, w); }
+
 // The same by radix-2 decimation-in-frequency stages whose twiddles tw(p, s) =
 // w^(p 2^s) the caller supplies (stage s pairs points p and p + 2^(K - s - 1) of its
 // blocks): as the first K stages of a longer transform, or its last ones.
-// The roundings of a butterfly's product are written out, so that they do not
-// depend on how the surrounding code is compiled.
 template <int K, int N, typename Tw>
 __device__ __forceinline__ void dft_stages(float2 (&x)[N], Tw tw) {
   using C = float2;
@@ -85,8 +91,7 @@ __device__ __forceinline__ void dft_stages(float2 (&x)[N], Tw tw) {
       for (int g = 0; g < R; g += 2 * h) {
         const C u = x[g + p], v = x[g + p + h];
         x[g + p] = cadd(u, v);
-        const C dl = csub(u, v);
-        x[g + p + h] = mk(__fmaf_rn(dl.x, w.x, -__fmul_rn(dl.y, w.y)), __fmaf_rn(dl.y, w.x, __fmul_rn(dl.x, w.y)));
+        x[g + p + h] = twiddled(csub(u, v), w);
       }
     }
   }

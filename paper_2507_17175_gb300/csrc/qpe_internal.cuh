@@ -135,6 +135,7 @@ struct FftArgs {
   int logb;    // B = 2^logb blocks
   int last;    // 1: no inter-pass twiddle
   int tw_sh;   // log2(N / transform length): a shard's local transform reads the N-point tables
+  int small;   // 1: a short transform's pass (fft_small_block)
   double scale;
 };
 
@@ -544,6 +545,7 @@ struct FftRound {  // one grouped QFT^-1 pass launch
   int item_off, nitems;
   int64_t blocks;
   size_t smem;
+  int small;  // all its items' FftArgs::small
 };
 
 struct BatchMeta {
@@ -702,11 +704,11 @@ template <typename C> int launch_init_grouped(const InitItem<C>* items, int nite
 template <typename C>
 int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, int dclass, int j, cudaStream_t s);
 template <typename C>
-int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, cudaStream_t s);
+int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, int small, cudaStream_t s);
 template <typename C> int launch_reduce_grouped(const RedItem<C>* items, int nitems, int64_t blocks, cudaStream_t s);
 // pass i's arguments, CTA count and shared memory; the plain histogram's CTA
 // count; the doubling GEMM's row / column tile for a target dimension d
-FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, size_t esize);
+FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, size_t esize, bool tiles = false);
 Digits fft_digits(const FftPlan& f);
 int64_t reduce_blocks(const Instance& in);
 void doubling_tile(int d, int* BM, int* BN);

@@ -465,6 +465,93 @@ __host__ __device__ constexpr int fft_k1(int logr) { return logr <= 4 ? logr : l
 template <typename C>
 constexpr int kFftThreads = sizeof(C) == 8 ? 256 : 128;
 
+// digit y of a pass at row offset b: the inter-pass twiddle, the scale, the store
+template <typename C>
+struct FftStore {
+  const C* __restrict__ tw_lo;
+  const C* __restrict__ tw_hi;
+  const FftArgs& a;
+  uint32_t lo_mask = (1u << a.htw) - 1u;
+  uint32_t rl_mask = (uint32_t)((int64_t(1) << (a.logr + a.logq - a.logd)) - 1);  // R L - 1
+  int esh = a.logb + a.tw_sh;
+  __device__ __forceinline__ void operator()(C v, C* dst, uint32_t b, int y) const {
+    if (!a.last) {  // omega_(RL)^(b y) = omega_N^(b y B); b y < R L <= N <= 2^30
+      const uint32_t e = ((b * (uint32_t)y) & rl_mask) << esh;
+      v = cmul(v, cmul(ld(tw_lo + (e & lo_mask)), ld(tw_hi + (e >> a.htw))));
+    }
+    if (a.scale != 1.0) v = cscale(v, (typename real_of<C>::type)a.scale);
+    dst[(int64_t)y << a.logq] = v;
+  }
+};
+
+// A pass of a short transform (the rule is in fft_pass_args): a CTA stages R rows of one
+// block x W columns (128 bytes, less where the rows are narrower) in shared memory and runs the
+// radix-2 stages there, three at a time in registers. With few CTAs a pass takes the
+// latency of one of them, and that is a matter of warps: at 8 points a thread there are up to
+// four times as many as at fft_tile's 32, and none work on padding.
+template <int K, typename C>
+__device__ __forceinline__ void fft_group(C* tile, const C* twp, int W, int row0, int logm, int logs, int logr) {
+  constexpr int RK = 1 << K;
+  C x[RK];
+#pragma unroll
+  for (int j = 0; j < RK; ++j) x[j] = tile[(row0 + (j << logs)) * W];
+#pragma unroll
+  for (int lt = 0; lt < K; ++lt) {
+    const int logh = logm - lt - 1;  // global half size h = 2^logh
+#pragma unroll
+    for (int j = 0; j < RK; ++j) {
+      const int hh = RK >> (lt + 1);
+      if (j & hh) continue;
+      const C u = x[j], v = x[j + hh];
+      x[j] = cadd(u, v);
+      x[j + hh] = twiddled(csub(u, v), twp[((row0 + (j << logs)) & ((1 << logh) - 1)) << (logr - logh - 1)]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < RK; ++j) tile[(row0 + (j << logs)) * W] = x[j];
+}
+
+template <typename C>
+__device__ __forceinline__ void fft_small_block(C* __restrict__ X, const C* __restrict__ tw_lo,
+                                                const C* __restrict__ tw_hi, const FftArgs& a, int64_t bid) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* tile = reinterpret_cast<C*>(smem_raw);
+  const int R = 1 << a.logr, W = 1 << a.logw, RW = R << a.logw;
+  C* twp = tile + RW;  // w_R^e, e < R / 2
+  const int slices_log = a.logq - a.logw;
+  const uint32_t q0 = (uint32_t)(bid & ((int64_t(1) << slices_log) - 1)) << a.logw;
+  C* base = X + ((bid >> slices_log) << (a.logr + a.logq)) + q0;
+  constexpr int V = 16 / (int)sizeof(C);  // elements per copy; W >= V: rows of at least 16 bytes
+  for (int i = threadIdx.x * V; i < RW; i += blockDim.x * V)
+    cp_async16(tile + i, base + ((int64_t)(i >> a.logw) << a.logq) + (i & (W - 1)));
+  cp_async_commit();
+  for (int e = threadIdx.x; e < (R >> 1); e += blockDim.x)
+    twp[e] = twiddle(tw_lo, tw_hi, a.htw, (int64_t)e << (a.n + a.tw_sh - a.logr));
+  cp_async_wait<0>();
+  __syncthreads();
+  // stages s0 .. s0 + K - 1 pair only the rows row0 + j 2^logs, j < 2^K, with each other
+  for (int s0 = 0; s0 < a.logr; s0 += 3) {
+    const int K = a.logr - s0 < 3 ? a.logr - s0 : 3;
+    const int logm = a.logr - s0, logs = logm - K;
+    for (int t = threadIdx.x; t < (RW >> K); t += blockDim.x) {
+      const int rest = t >> a.logw;
+      const int row0 = ((rest >> logs) << logm) + (rest & ((1 << logs) - 1));
+      C* col = tile + (t & (W - 1));
+      switch (K) {
+        case 1: fft_group<1>(col, twp, W, row0, logm, logs, a.logr); break;
+        case 2: fft_group<2>(col, twp, W, row0, logm, logs, a.logr); break;
+        default: fft_group<3>(col, twp, W, row0, logm, logs, a.logr); break;
+      }
+    }
+    __syncthreads();
+  }
+  const FftStore<C> store{tw_lo, tw_hi, a};
+  for (int i = threadIdx.x; i < RW; i += blockDim.x) {
+    const int r = i >> a.logw, w = i & (W - 1);
+    store(tile[i], base + w, (q0 + (uint32_t)w) >> a.logd, (int)(__brev((uint32_t)r) >> (32 - a.logr)));
+  }
+}
+
 template <typename C, int K1, int K2>
 __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict__ tw_lo, const C* __restrict__ tw_hi,
                                          const FftArgs& a, int64_t bid) {
@@ -492,31 +579,22 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
     blk = bid << logg;
     q0 = 0;
   }
-  const int gn = (int)((int64_t(1) << a.logb) - blk < (1 << logg) ? (int64_t(1) << a.logb) - blk : 1 << logg);
   C* base = X + (blk << (K1 + K2 + a.logq)) + q0;
   const int tid = threadIdx.x;
 
-  // rows n1 R2 + n2 of column (g, w): w fastest, then n2, then g
-  const int T1 = R2 << a.logc;
+  // rows n1 R2 + n2 of column (g, w): w fastest, then n2, then g < gn, the blocks there are
+  // (a whole tile's unless the transform is shorter than one)
+  const int64_t left = (int64_t(1) << a.logb) - blk;
+  const int gn = left < (1 << logg) ? (int)left : 1 << logg;
+  const int T1 = gn << (K2 + logw);
   C x[R1];
   auto load = [&](int t) {
     const int w = t & (W - 1), n2 = (t >> logw) & (R2 - 1), g = t >> (logw + K2);
     const C* src = base + ((int64_t)g << (K1 + K2 + a.logq)) + ((int64_t)n2 << a.logq) + w;
 #pragma unroll
-    for (int j = 0; j < R1; ++j) x[j] = g < gn ? src[(int64_t)(j * R2) << a.logq] : mk((R_t)0, (R_t)0);
+    for (int j = 0; j < R1; ++j) x[j] = src[(int64_t)(j * R2) << a.logq];
   };
-  // digit y of column (g, w): the inter-pass twiddle, the scale, the store
-  const uint32_t lo_mask = (1u << a.htw) - 1u;
-  const uint32_t rl_mask = (uint32_t)((int64_t(1) << (K1 + K2 + a.logq - a.logd)) - 1);  // R L - 1
-  const int esh = a.logb + a.tw_sh;
-  auto store = [&](C v, C* dst, uint32_t b, int y) {
-    if (!a.last) {  // omega_(RL)^(b y) = omega_N^(b y B); b y < R L <= N <= 2^30
-      const uint32_t e = ((b * (uint32_t)y) & rl_mask) << esh;
-      v = cmul(v, cmul(ld(tw_lo + (e & lo_mask)), ld(tw_hi + (e >> a.htw))));
-    }
-    if (a.scale != 1.0) v = cscale(v, (R_t)a.scale);
-    dst[(int64_t)y << a.logq] = v;
-  };
+  const FftStore<C> store{tw_lo, tw_hi, a};
   if (tid < T1) load(tid);
   if constexpr (K2 > 0 || kStages) {
     for (int e = tid; e < (kStages ? R1 * R2 / 2 : R1 * R2); e += NT)
@@ -531,12 +609,10 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
     else
       dft_k<C, K1, R1>(x);
     if constexpr (K2 == 0) {
-      if (g < gn) {
-        C* dst = base + ((int64_t)g << (K1 + a.logq)) + w;
-        const uint32_t b = (q0 + (uint32_t)w) >> a.logd;
+      C* dst = base + ((int64_t)g << (K1 + a.logq)) + w;
+      const uint32_t b = (q0 + (uint32_t)w) >> a.logd;
 #pragma unroll
-        for (int k = 0; k < R1; ++k) store(x[k], dst, b, k);
-      }
+      for (int k = 0; k < R1; ++k) store(x[k], dst, b, k);
     } else {
       C* dst = tile + (g * R1) * kld + (n2 << logw) + w;
 #pragma unroll
@@ -545,10 +621,9 @@ __device__ __forceinline__ void fft_tile(C* __restrict__ X, const C* __restrict_
   }
   if constexpr (K2 > 0) {
     __syncthreads();
-    const int T2 = R1 << a.logc;
+    const int T2 = gn << (K1 + logw);
     for (int t = tid; t < T2; t += NT) {  // w fastest, then k1, then g
       const int w = t & (W - 1), k1 = (t >> logw) & (R1 - 1), g = t >> (logw + K1);
-      if (g >= gn) break;
       const C* src = tile + (g * R1 + k1) * kld + w;
       C z[R2];
 #pragma unroll
@@ -588,12 +663,28 @@ __global__ void __launch_bounds__(kFftThreads<C>, 2) fft_pass_kernel(C* __restri
   fft_pass_block<C>(X, tw_lo, tw_hi, a, blockIdx.x);
 }
 
+constexpr int kFftSmallThreads = 256;
+template <typename C>
+__global__ void __launch_bounds__(kFftSmallThreads) fft_small_kernel(C* __restrict__ X, const C* __restrict__ tw_lo,
+                                                                     const C* __restrict__ tw_hi, FftArgs a) {
+  pdl_begin();
+  fft_small_block<C>(X, tw_lo, tw_hi, a, blockIdx.x);
+}
+
 // One QFT^-1 pass of every listed instance (each item its own pass arguments).
 template <typename C>
 __global__ void __launch_bounds__(kFftThreads<C>, 2) fft_pass_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
   pdl_begin();
   const int i = find_item(items, nitems, blockIdx.x);
   fft_pass_block<C>(items[i].X, items[i].lo, items[i].hi, items[i].a, blockIdx.x - items[i].tile0);
+}
+template <typename C>
+__global__ void __launch_bounds__(kFftSmallThreads)
+    fft_small_grouped_kernel(const FftItem<C>* __restrict__ items, int nitems) {
+  pdl_begin();
+  const int i = find_item(items, nitems, blockIdx.x);
+  const FftItem<C> it = items[i];
+  fft_small_block<C>(it.X, it.lo, it.hi, it.a, blockIdx.x - it.tile0);
 }
 
 // --------------------------------------------------------------- reduce
@@ -1276,7 +1367,8 @@ int64_t fft_position_to_y(const FftPlan& f, int nmeas, int64_t p) {
 }
 
 constexpr int kFftSmemMax = 96 * 1024;  // 64 KiB of tile, at most 16 of padding and 8 of twiddles
-FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, size_t esize) {
+// tiles: fft_tile for short transforms too
+FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, size_t esize, bool tiles) {
   const FftPass& p = in.fft.p[i];
   FftArgs a;
   a.logr = p.logr;
@@ -1293,6 +1385,19 @@ FftArgs fft_pass_args(const Instance& in, int i, int64_t* blocks, size_t* smem, 
   // that are taken from several consecutive blocks
   const int64_t points = p.B * p.Q << p.logr;
   a.logc = ilog2((int64_t)(128 / esize));
+  // Short transforms take fft_small_block in passes of four bits or more: fewer than 2^18
+  // points in complex128, 2^17 in complex64. Times of all passes, fft_small_block against
+  // fft_tile, us: complex128 2^10 points, one pass of 7 bits 14.3 against 20.1, 2^12 points, one of 9
+  // bits 49 against 55; 2^17 points, 7 + 7 bits 28.6 against 34.8; 2^18 points, 7 + 7 bits 47 both, 9 + 8
+  // bits 85 against 80; 3 bits 9.6 against 8.2. complex64 2^13 .. 2^17 points, one pass of 9 bits 10 against
+  // 12; 2^17 points, 8 + 8 bits 13.1 against 12.2; 2^18 points, 9 + 8 bits 19.3 against 17.4.
+  a.small = !tiles && a.logr >= 4 && points < (esize == 16 ? int64_t(1) << 18 : int64_t(1) << 17);
+  if (a.small) {
+    a.logw = a.logc = std::min(a.logq, a.logc);
+    *blocks = points >> (a.logr + a.logc);
+    *smem = ((((size_t)1 << a.logc) << a.logr) + ((size_t)1 << a.logr) / 2) * esize;
+    return a;
+  }
   while (((int64_t)esize << (a.logr + a.logc + 1)) <= 64 * 1024 && (points >> (a.logr + a.logc + 1)) >= 4 * 152) ++a.logc;
   a.logw = std::min(a.logq, a.logc);
   *blocks = std::max<int64_t>(1, points >> (a.logr + a.logc));
@@ -1313,8 +1418,10 @@ int launch_fft(const Instance& in, char* ws, cudaStream_t s) {
     int64_t blocks = 0;
     size_t smem = 0;
     const FftArgs a = fft_pass_args(in, i, &blocks, &smem, sizeof(C));
-    if (launch_k(fft_pass_kernel<C>, dim3((unsigned)blocks), dim3(kFftThreads<C>), smem, s, X, lo, hi, a) != cudaSuccess)
-      return -1;
+    const cudaError_t e =
+        a.small ? launch_k(fft_small_kernel<C>, dim3((unsigned)blocks), dim3(kFftSmallThreads), smem, s, X, lo, hi, a)
+                : launch_k(fft_pass_kernel<C>, dim3((unsigned)blocks), dim3(kFftThreads<C>), smem, s, X, lo, hi, a);
+    if (e != cudaSuccess) return -1;
     ++launches;
   }
   return launches;
@@ -1372,12 +1479,13 @@ int launch_doubling_grouped(const DblItem<C>* items, int nitems, int64_t tiles, 
 }
 
 template <typename C>
-int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, cudaStream_t s) {
+int launch_fft_grouped(const FftItem<C>* items, int nitems, int64_t blocks, size_t smem, int small, cudaStream_t s) {
   if (nitems <= 0) return 0;
-  return launch_k(fft_pass_grouped_kernel<C>, dim3((unsigned)blocks), dim3(kFftThreads<C>), smem, s, items, nitems) ==
-                 cudaSuccess
-             ? 1
-             : -1;
+  const dim3 grid((unsigned)blocks);
+  const cudaError_t e =
+      small ? launch_k(fft_small_grouped_kernel<C>, grid, dim3(kFftSmallThreads), smem, s, items, nitems)
+            : launch_k(fft_pass_grouped_kernel<C>, grid, dim3(kFftThreads<C>), smem, s, items, nitems);
+  return e == cudaSuccess ? 1 : -1;
 }
 
 template <typename C>
@@ -1458,15 +1566,15 @@ int launch_unpermute(const Instance& in, const char* ws, void* out, cudaStream_t
 cudaError_t configure_kernels() {
   cudaError_t e = configure_level_kernels();
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fft_pass_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fft_pass_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fft_pass_grouped_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           kFftSmemMax);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(fft_pass_grouped_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kFftSmemMax);
+  const void* fft[] = {(const void*)fft_pass_kernel<float2>,          (const void*)fft_pass_kernel<double2>,
+                       (const void*)fft_pass_grouped_kernel<float2>,  (const void*)fft_pass_grouped_kernel<double2>,
+                       (const void*)fft_small_kernel<float2>,         (const void*)fft_small_kernel<double2>,
+                       (const void*)fft_small_grouped_kernel<float2>, (const void*)fft_small_grouped_kernel<double2>};
+  for (const void* k : fft) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 template int launch_sweep<float2>(const Instance&, char*, bool, cudaStream_t, int);
@@ -1477,7 +1585,7 @@ template int launch_reduce<float2>(const Instance&, char*, cudaStream_t);
 #define QPE_GROUPED_INST(C)                                                                             \
   template int launch_init_grouped<C>(const InitItem<C>*, int, cudaStream_t);                          \
   template int launch_doubling_grouped<C>(const DblItem<C>*, int, int64_t, int, int, cudaStream_t);    \
-  template int launch_fft_grouped<C>(const FftItem<C>*, int, int64_t, size_t, cudaStream_t);           \
+  template int launch_fft_grouped<C>(const FftItem<C>*, int, int64_t, size_t, int, cudaStream_t);      \
   template int launch_reduce_grouped<C>(const RedItem<C>*, int, int64_t, cudaStream_t);
 QPE_GROUPED_INST(float2)
 QPE_GROUPED_INST(double2)
