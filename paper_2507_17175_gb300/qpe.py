@@ -304,6 +304,13 @@ def _order_after_current(stream, device):
         stream.wait_stream(current)
 
 
+def _order_current_after(stream, device):
+    """What the current stream is given from here on waits for ``stream``."""
+    current = _other_current(stream, device)
+    if current is not None:
+        current.wait_stream(stream)
+
+
 class Plan:
     """One QPE problem bound to a torch-allocated workspace and stream."""
 
@@ -385,6 +392,8 @@ class Plan:
         if want_hist and out is None:
             out = np.empty(self.N, dtype=np.float64)
         ptr, dev = (0, 0) if out is None else _ptr(out)
+        if dev:
+            _order_after_current(self.stream, self.device)
         self._check(_lib.qpe_probs(self._h, instance, ptr or None, ctypes.byref(am), ctypes.byref(pa),
                                    ctypes.byref(pm), dev), "qpe_probs")
         return out, am.value, pa.value, pm.value
@@ -393,7 +402,11 @@ class Plan:
         if out is None:
             out = np.empty((self.N, self.d), dtype=self.state_dtype)
         ptr, dev = _ptr(out)
+        if dev:
+            _order_after_current(self.stream, self.device)
         self._check(_lib.qpe_state(self._h, instance, ptr, dev), "qpe_state")
+        if dev:  # enqueued only: what the current stream does with it comes after
+            _order_current_after(self.stream, self.device)
         return out
 
     def load_state(self, S, instance: int = 0):
@@ -573,6 +586,8 @@ class BatchedPlan(Plan):
         if want_hist and out is None:
             out = np.empty(1 << nmeas, dtype=np.float64)
         ptr, dev = (0, 0) if out is None else _ptr(out)
+        if dev:
+            _order_after_current(self.stream, self.device)
         self._check(_lib.qpe_probs(self._h, instance, ptr or None, ctypes.byref(am), ctypes.byref(pa),
                                    ctypes.byref(pm), dev), "qpe_probs")
         return out, am.value, pa.value, pm.value
@@ -582,5 +597,9 @@ class BatchedPlan(Plan):
         if out is None:
             out = np.empty((1 << nmeas, 1 << nmat), dtype=self.state_dtype)
         ptr, dev = _ptr(out)
+        if dev:
+            _order_after_current(self.stream, self.device)
         self._check(_lib.qpe_state(self._h, instance, ptr, dev), "qpe_state")
+        if dev:  # enqueued only: what the current stream does with it comes after
+            _order_current_after(self.stream, self.device)
         return out

@@ -86,6 +86,26 @@ def test_no_wait_on_the_same_stream_or_while_it_is_captured(recorded, call):
     assert not any(entry[0] == "wait" for entry in log)
 
 
+OUTPUTS = {
+    "probs": lambda p: p.probs(_tensor(4, dtype=torch.float64)),
+    "state": lambda p: p.state(_tensor(4, 2, dtype=torch.complex64)),
+    "batched_probs": lambda p: p.probs(0, _tensor(4, dtype=torch.float64)),
+    "batched_state": lambda p: p.state(0, _tensor(4, 2, dtype=torch.complex64)),
+}
+
+
+@pytest.mark.parametrize("call", OUTPUTS)
+def test_device_outputs_are_ordered_with_the_current_stream(recorded, call):
+    """A buffer the current stream still reads is not overwritten, and what that stream
+    does next with a state that is only enqueued waits for it (qpe_probs returns when
+    the bins are there)."""
+    make, log, _ = recorded
+    OUTPUTS[call](make(qpe.BatchedPlan if call.startswith("batched") else qpe.Plan))
+    at = log.index(("qpe_" + call.split("_")[-1],))
+    assert ("wait", OWN, CURRENT) in log[:at]
+    assert ("wait", CURRENT, OWN) in log[at:] or call.endswith("probs")
+
+
 def test_host_inputs_do_not_wait(recorded):
     make, log, _ = recorded
     plan = make()
@@ -136,3 +156,33 @@ def test_inputs_still_being_computed(batched):
     plan.run()
     for got, ref in zip(bins(), want):
         np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.gpu
+def test_outputs_still_being_read():
+    """The current stream's late copy of the last run's outputs is not overtaken by the next
+    run's, and its copies of the next outputs see them whole."""
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    Us = [torch.linalg.qr(torch.randn((4, 4), generator=gen, dtype=torch.complex128, device="cuda"))[0].contiguous()
+          for _ in range(2)]
+    plan = qpe.Plan(2, 16, qpe.FP64, qpe.FLAG_GRAPH | qpe.FLAG_PLAIN)
+    filler = torch.eye(8192, device="cuda")
+    hist = torch.empty(plan.N, dtype=torch.float64, device="cuda")
+    state = torch.empty((plan.N, plan.d), dtype=torch.complex128, device="cuda")
+
+    def run(U):
+        plan.load(U, U[:, 0].contiguous())
+        plan.run()
+        plan.probs(hist)
+        plan.state(state)
+        return hist.clone(), state.clone()
+
+    want = [run(U) for U in Us]
+    torch.cuda.synchronize()
+    run(Us[0])
+    torch.cuda.synchronize()
+    filler @ filler  # the copies below come late
+    got = [(hist.clone(), state.clone()), run(Us[1])]
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        assert torch.equal(g[0], w[0]) and torch.equal(g[1], w[1])
