@@ -295,13 +295,18 @@ def _other_current(stream, device):
     return current
 
 
-def _order_after_current(stream, device):
+def _order_after_current(stream, device, *tensors):
     """What is enqueued on ``stream`` from here on waits for the current stream:
     a caller's tensors are written there, and torch hands out memory whose last
-    user there may still be running."""
+    user there may still be running. ``tensors``: read or written on ``stream``
+    after the call returns; torch keeps their memory until ``stream`` is past that,
+    however early they are dropped."""
     current = _other_current(stream, device)
     if current is not None:
         stream.wait_stream(current)
+        for t in tensors:
+            if getattr(t, "is_cuda", False):
+                t.record_stream(stream)
 
 
 def _order_current_after(stream, device):
@@ -327,13 +332,19 @@ class Plan:
             stream = torch.cuda.Stream(device=self.device) if (flags & FLAG_GRAPH) else \
                 torch.cuda.current_stream(self.device)
         self.stream = stream
+        self._bind(workspace)
+
+    # -------------------------------------------------------------- helpers
+    def _bind(self, workspace):
+        """Bind to ``workspace`` (from torch if None), whose memory torch keeps until the
+        plan's stream is done with it, also when the plan is dropped before."""
+        import torch
         if workspace is None:
             workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = workspace
-        _order_after_current(stream, self.device)
-        self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
+        _order_after_current(self.stream, self.device, workspace)
+        self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, self.stream.cuda_stream), "qpe_bind")
 
-    # -------------------------------------------------------------- helpers
     def _check(self, st: int, what: str):
         if st != OK:
             msg = _lib.qpe_last_error(self._h).decode() if self._h else ""
@@ -362,7 +373,7 @@ class Plan:
         if du != dp:
             raise ValueError("U and psi must both be host or both be device buffers")
         if du:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self.stream, self.device, U, psi)
         self._keep = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, self.nmat, self.nmeas, du), "qpe_load")
 
@@ -414,7 +425,7 @@ class Plan:
             S = np.ascontiguousarray(S, dtype=self.state_dtype)
         ptr, dev = _ptr(S)
         if dev:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self.stream, self.device, S)
         self._keep_state = S
         self._check(_lib.qpe_load_state(self._h, instance, ptr, dev), "qpe_load_state")
 
@@ -475,11 +486,7 @@ class ShardedPlan(Plan):
             stream = torch.cuda.Stream(device=self.device) if (flags & FLAG_GRAPH) else \
                 torch.cuda.current_stream(self.device)
         self.stream = stream
-        if workspace is None:
-            workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
-        self.workspace = workspace
-        _order_after_current(stream, self.device)
-        self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
+        self._bind(workspace)
 
     def probs(self, out=None, instance: int = 0, want_hist: bool = True):
         if want_hist and out is None:
@@ -559,12 +566,8 @@ class BatchedPlan(Plan):
             stream = torch.cuda.Stream(device=self.device) if (flags & FLAG_GRAPH) else \
                 torch.cuda.current_stream(self.device)
         self.stream = stream
-        if workspace is None:
-            workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
-        self.workspace = workspace
         self._keep_inputs = {}
-        _order_after_current(stream, self.device)
-        self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, stream.cuda_stream), "qpe_bind")
+        self._bind(workspace)
 
     def load(self, instance: int, U, psi):
         nmat, nmeas = self.shapes[instance]
@@ -574,7 +577,7 @@ class BatchedPlan(Plan):
         pu, du = _ptr(U)
         pp, dp = _ptr(psi)
         if du:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self.stream, self.device, U, psi)
         self._keep_inputs[instance] = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, nmat, nmeas, du), "qpe_load")
 

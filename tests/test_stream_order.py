@@ -23,6 +23,9 @@ class _Tensor(torch.Tensor):
     """A host tensor that says it lies on the GPU."""
     is_cuda = True
 
+    def record_stream(self, stream):
+        stream.log.append(("record", stream.cuda_stream, self.data_ptr()))
+
 
 class _Lib:
     def __init__(self, log):
@@ -74,6 +77,24 @@ def test_device_inputs_are_ordered_after_the_current_stream(recorded, call):
     INPUTS[call](make(qpe.BatchedPlan if call.startswith("batched") else qpe.Plan))
     enqueue = ("qpe_load_state",) if call == "load_state" else ("qpe_load",)
     assert ("wait", OWN, CURRENT) in log[:log.index(enqueue)]
+
+
+@pytest.mark.parametrize("call", INPUTS)
+def test_memory_of_dropped_inputs_waits_for_the_copy(recorded, call):
+    make, log, _ = recorded
+    INPUTS[call](make(qpe.BatchedPlan if call.startswith("batched") else qpe.Plan))
+    assert sum(entry[:2] == ("record", OWN) for entry in log) == (1 if call == "load_state" else 2)
+
+
+@pytest.mark.parametrize("cls,args", [(qpe.Plan, (1, 2, qpe.C64_FP32, qpe.FLAG_GRAPH)),
+                                      (qpe.ShardedPlan, (1, 2, qpe.C64_FP32, qpe.FLAG_GRAPH, 0, 2)),
+                                      (qpe.BatchedPlan, ([(1, 2)], qpe.C64_FP32, qpe.FLAG_GRAPH))])
+def test_workspace_of_a_dropped_plan_waits_for_its_run(recorded, cls, args):
+    _, log, _ = recorded
+    ws = _tensor(64, dtype=torch.uint8)
+    cls(*args, stream=_Stream(OWN, log), workspace=ws)
+    assert ("record", OWN, ws.data_ptr()) in log
+    assert log.index(("wait", OWN, CURRENT)) < log.index(("qpe_bind",))
 
 
 @pytest.mark.parametrize("call", INPUTS)
