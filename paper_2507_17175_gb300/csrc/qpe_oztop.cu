@@ -26,15 +26,15 @@
 // GB300 issues an FP64 instruction at 1/32 of the rate of a 32-bit integer
 // one, so the epilogue stays in 64-bit fixed point up to the sums of |X|^2: the drain
 // reads each accumulator as an int (a magic-number addition in FP32), forms
-// W = floor(E / 2^10) (|W| < 2^57 + 1, units 2^(tau + sigma - 52)),
+// W = floor(E / 2^9) (|W| < 2^58 + 1, units 2^(tau + sigma - 53)),
 // multiplies by the twiddles held in Q61 (round(w 2^61), split at bit 31 into
 // int32 halves so that every partial product is one 32 x 32 -> 64-bit
 // multiply-add; at most 3 units off), runs the 8-point DFT on the integers
-// (|X| < 8 sqrt(2) 2^57 < 2^61; the factor cos(pi / 4) also in Q61), sums |X|^2
-// exactly in integers (OtSquares; the unit goes into the histogram's scale once
+// (|X| < 8 sqrt(2) 2^58 < 2^62; the factor cos(pi / 4) also in Q61), sums |X|^2
+// in integers (OtSquares; the unit goes into the histogram's scale once
 // per tile) or, in a lower level (MODE 0), stores X in FP64 (the hardware
 // conversion, rounded to nearest; the unit's power of two goes into the exponent
-// bits). The fixed point's truncations are a few units, 2^-55 of the pencil's
+// bits). The fixed point's truncations are a few units, 2^-56 of the pencil's
 // bound |T| < 2^(tau + sigma + 5), below the contraction's own error. The sums
 // over the warps and the readout run in FP64. Top level at Nmeas 24: 4.0 ms with
 // its lower levels before the MMA warp ran converged, 3.2 so (2.48 ms alone).
@@ -58,6 +58,7 @@
 //               then the sums of |X|^2 (the four warps' meet as doubles through
 //               tensor memory columns 448-495) or the store of X in FP64.
 // Every wait is a bounded mbarrier wait; an expired wait sets QPE_ERR_TIMEOUT.
+#include "qpe_fixed.cuh"
 #include "qpe_internal.cuh"
 #include "qpe_tcgen05.cuh"
 
@@ -95,30 +96,6 @@ __device__ __forceinline__ double ot_scale2(double v, int e) {
   const long long b = __double_as_longlong(v);
   const int E = (int)((b >> 52) & 0x7ff);
   return (E == 0 || E + e <= 0) ? 0.0 : __longlong_as_double(b + ((long long)e << 52));
-}
-
-// A weight accumulator (an exact integer |acc| < 2^22 in FP32) plus 1.5 2^23
-// in FP32 is exact and has the bits acc + M, M = 0x4B400000.
-__device__ __forceinline__ uint32_t ot_acc_bits(uint32_t u) {
-  return __float_as_uint(__fadd_rn(__uint_as_float(u), 12582912.0f));
-}
-
-// The drain's fixed point W = floor(E / 2^10) of one T component from its
-// seven weight sums, E = sum_w acc_w 2^(8 (6 - w)), T = 2^(tau + sigma - 62) E.
-// With b_w = acc_w + M, the low part acc_5 2^8 + acc_6 = b_5 2^8 + b_6 - 257 M
-// (exact in int32), and the rest sum_(w<5) b_w 2^(8 (6 - w) - 10) minus
-// M sum_(w<5) 2^(8 (6 - w) - 10), modulo 2^64 (W itself fits).
-__device__ __forceinline__ long long ot_weights_fix(uint32_t u0, uint32_t u1, uint32_t u2, uint32_t u3, uint32_t u4,
-                                                    uint32_t u5, uint32_t u6) {
-  constexpr unsigned long long kMW = 0xe2e2e2e2d0000000ull;  // M (2^38 + 2^30 + 2^22 + 2^14 + 2^6) mod 2^64
-  const int r = (int)(ot_acc_bits(u5) * 256u + ot_acc_bits(u6) - 0x8b400000u) >> 10;  // 257 M mod 2^32
-  unsigned long long w = (unsigned long long)(long long)r - kMW;
-  w += (unsigned long long)ot_acc_bits(u4) * 64u;
-  w += (unsigned long long)ot_acc_bits(u3) * 16384u;
-  w += (unsigned long long)ot_acc_bits(u2) * 4194304u;
-  w += (unsigned long long)ot_acc_bits(u1) * 1073741824u;
-  w += (unsigned long long)(ot_acc_bits(u0) * 64u) << 32;
-  return (long long)w;
 }
 
 // (wr + i wi) (qr + i qi) 2^-61 for a twiddle in Q61 (q = round(w 2^61)),
@@ -184,40 +161,6 @@ __device__ __forceinline__ void ot_dft8_fix(long long (&x)[16]) {
   t = x[6]; x[6] = x[12]; x[12] = t;
   t = x[7]; x[7] = x[13]; x[13] = t;
 }
-
-// Sums of squares of the fixed-point X (|X| < 2^60.6; its lowest bit, below the
-// fixed point's own few units of error, is dropped): with X = A 2^32 + 2 b, b in
-// [-2^30, 2^30), X^2 = A^2 2^64 + A b 2^34 + b^2 4, each part summed exactly by one
-// 32 x 32 + 64-bit multiply-add (|A| < 2^28.7; eight squares stay below 2^63).
-// GB300 issues FP64 at 2 lanes a clock and SM, so a conversion and an FP64 FMA for
-// every value kept the FP64 pipe 76% busy and were what the top level waited
-// for; here the FP64 work is one value per bin and drain thread.
-struct OtSquares {
-  unsigned long long hh = 0, ll = 0;
-  long long hl = 0;
-  __device__ __forceinline__ void add(long long x) {
-    const uint32_t lo = (uint32_t)x;
-    const int A = (int)(x >> 32) + (int)(lo >> 31);
-    const int b = (int)lo >> 1;
-    hh += (unsigned long long)((long long)A * A);
-    hl += (long long)A * b;
-    ll += (unsigned long long)((long long)b * b);
-  }
-  // the sum as a double, by integer operations: all drain warps reach this at the
-  // end of a tile, and five FP64 operations a bin there took 10,000 clocks of the
-  // SM during which no accumulator was read
-  __device__ __forceinline__ double value() const {
-    const unsigned long long mid = (unsigned long long)hl << 34, low = ll << 2;
-    const unsigned long long lo = low + mid;
-    const unsigned long long hi = hh + (unsigned long long)(hl >> 30) + (ll >> 62) + (lo < low ? 1 : 0);
-    const unsigned long long top = hi ? hi : lo;
-    if (top == 0) return 0.0;
-    const int n = __clzll((long long)top);
-    const unsigned long long frac = (hi && n) ? (hi << n) | (lo >> (64 - n)) : top << n;  // leading bit at 63
-    const unsigned long long exp = (unsigned long long)(1023 + 63 + (hi ? 64 : 0) - n - 1);  // less the leading one
-    return __longlong_as_double((long long)((exp << 52) + (frac >> 11) + ((frac >> 10) & 1)));
-  }
-};
 
 // better() for a bin v >= 0 (or NaN, which is never better): nonnegative doubles
 // order as their bits, off the FP64 pipe
@@ -574,8 +517,8 @@ __global__ void __launch_bounds__(kOtThreads, 1) level_oz_kernel(OzTopArgs a) {
         break;
       }
       const int4* tw = twS + (tb * kOtRows + row) * (kOtL - 1);
-      // X in units of 2^(tau + sigma - 52) (the fixed point below)
-      const int e2 = tauS[tb * kOtRows + row] - 22;
+      // X in units of 2^(tau + sigma - 62 + kOtFix) (the fixed point below)
+      const int e2 = tauS[tb * kOtRows + row] - 32 + kOtFix;
       const int64_t jt = t * kOtRows + row;  // local pencil index
       OtSquares sq2[kOtL];
       for (int c = par; c < kOtChunks; c += 2, ++uses) {
