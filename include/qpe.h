@@ -319,7 +319,9 @@ qpe_status qpe_probs(qpe_plan_t plan, int32_t instance, double* probs, int64_t* 
  * natural row order: after SWEEP, row m = 2^(-n/2) U^m psi; after FFT, row y
  * is the final statevector (the paper's output file, Sec. 3). Host output
  * synchronises and reorders on the host; device output is reordered by a
- * kernel on the stream. After a fused qpe_run the final state exists only
+ * kernel on the stream. A device output lies on a boundary of its real type
+ * (8 bytes for complex128, 4 for complex64; QPE_ERR_ARG otherwise); one of 16
+ * bytes is the fastest. After a fused qpe_run the final state exists only
  * with QPE_FLAG_KEEP_STATE (QPE_ERR_STATE otherwise).
  */
 qpe_status qpe_state(qpe_plan_t plan, int32_t instance, void* out, int32_t ptr_is_device);
@@ -404,11 +406,12 @@ typedef struct {
  *
  * final_state: device pointer to the N x d final statevector in natural row
  * order (complex128 for QPE_FP64, complex64 for the other precisions), as
- * qpe_state returns it. Outputs, device pointers owned by the caller: probs
+ * qpe_state returns it, on a boundary of its real type (of 16 bytes: the
+ * fastest). Outputs, device pointers owned by the caller: probs
  * (N doubles, P[y] = sum_t |X[y][t]|^2) and *readout. Enqueued on
  * cuda_stream (a cudaStream_t, NULL = legacy default stream); no host
  * synchronisation. Nmeas above 21 is rejected with QPE_ERR_WORKSPACE (the
- * largest histogram of a call without a workspace); bad pointers or
+ * largest histogram of a call without a workspace); bad or misaligned pointers or
  * shapes with QPE_ERR_ARG. The first call on each device looks up the
  * scratch's device address (cudaGetSymbolAddress); make that first call
  * outside any stream capture. All calls on a device share the scratch: two

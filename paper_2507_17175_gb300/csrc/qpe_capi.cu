@@ -1426,6 +1426,8 @@ qpe_status qpe_state(qpe_plan_t p, int32_t instance, void* out, int32_t ptr_is_d
     return QPE_OK;
   }
   if (ptr_is_device) {
+    if (reinterpret_cast<uintptr_t>(out) % (c64 ? 4 : 8) != 0)
+      return fail(p, QPE_ERR_ARG, "a device state must lie on a boundary of its real type");
     const int r = c64 ? qpe::launch_unpermute<float2>(*in, p->ws, out, p->stream)
                       : qpe::launch_unpermute<double2>(*in, p->ws, out, p->stream);
     if (r < 0) return cuda_fail(p, cudaGetLastError(), "unpermute kernel");

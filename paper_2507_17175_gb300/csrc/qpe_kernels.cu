@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "qpe_dft.cuh"
 #include "qpe_internal.cuh"
 
@@ -1045,17 +1047,18 @@ __global__ void __launch_bounds__(256) unpermute_kernel(const float4* __restrict
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = X[(y_to_pos(g, n, i >> vr) << vr) | (i & mask)];
 }
-// the same element by element, for an output on an 8-byte boundary
-template <typename C>
-__global__ void unpermute_elements_kernel(const C* __restrict__ X, C* __restrict__ out, int64_t N, int logd, int n,
+// the same in elements of E (2^loge a row), for an output on a smaller boundary: of 8
+// bytes, or of a float's 4
+template <typename E>
+__global__ void unpermute_elements_kernel(const E* __restrict__ X, E* __restrict__ out, int64_t N, int loge, int n,
                                           Digits g) {
   pdl_begin();
-  const int64_t total = N << logd;
-  const int64_t dmask = (int64_t(1) << logd) - 1;
+  const int64_t total = N << loge;
+  const int64_t emask = (int64_t(1) << loge) - 1;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t y = i >> logd;
-    out[i] = X[(y_to_pos(g, n, y) << logd) | (i & dmask)];
+    const int64_t y = i >> loge;
+    out[i] = X[(y_to_pos(g, n, y) << loge) | (i & emask)];
   }
 }
 
@@ -1548,12 +1551,18 @@ int launch_finalize(const Instance& in, char* ws, int count, cudaStream_t s) {
 template <typename C>
 int launch_unpermute(const Instance& in, const char* ws, void* out, cudaStream_t s) {
   const Digits g = digits_of(in.fft);
-  if (reinterpret_cast<uintptr_t>(out) % 16 != 0)
-    return launch_k(unpermute_elements_kernel<C>, dim3(grid_for(in.N * in.d, 256)), dim3(256), 0, s,
-                    reinterpret_cast<const C*>(ws + in.off_state), reinterpret_cast<C*>(out), in.N, in.nmat, in.nmeas,
-                    g) == cudaSuccess
+  auto elements = [&](auto kernel, auto* dst, size_t size) {
+    using E = std::remove_pointer_t<decltype(dst)>;
+    const int loge = ilog2(in.d * (int64_t)(sizeof(C) / size));
+    return launch_k(kernel, dim3(grid_for(in.N << loge, 256)), dim3(256), 0, s,
+                    reinterpret_cast<const E*>(ws + in.off_state), dst, in.N, loge, in.nmeas, g) == cudaSuccess
                ? 1
                : -1;
+  };
+  if (reinterpret_cast<uintptr_t>(out) % 8 != 0)
+    return elements(unpermute_elements_kernel<float>, static_cast<float*>(out), sizeof(float));
+  if (reinterpret_cast<uintptr_t>(out) % 16 != 0)
+    return elements(unpermute_elements_kernel<float2>, static_cast<float2*>(out), sizeof(float2));
   const int vr = in.nmat - (sizeof(C) == 8 ? 1 : 0);  // a row is 2^vr pieces of 16 bytes
   return launch_k(unpermute_kernel, dim3(grid_for(in.N << vr, 8 * 256)), dim3(256), 0, s,
                   reinterpret_cast<const float4*>(ws + in.off_state), reinterpret_cast<float4*>(out), in.N, vr, in.nmeas,

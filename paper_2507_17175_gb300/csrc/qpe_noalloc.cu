@@ -91,12 +91,18 @@ __device__ __forceinline__ double unpack(const RowSum& r) {
 
 // VPL 16-byte vectors a lane, LANES lanes a row (of at most 256 columns)
 template <int VPL, int LANES>
-__device__ __forceinline__ RowSum row_sum(const float2* __restrict__ row, int sub, bool vec16) {
+__device__ __forceinline__ RowSum row_sum(const float2* __restrict__ row, int sub, int bytes) {
   float4 v[VPL];
-  if (vec16) {
+  if (bytes == 16) {
 #pragma unroll
     for (int k = 0; k < VPL; ++k) v[k] = __ldcs(reinterpret_cast<const float4*>(row) + sub + k * LANES);
-  } else {  // a state on an 8-byte boundary
+  } else if (bytes == 4) {  // a state on a boundary of 4 bytes
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) {
+      const float* f = reinterpret_cast<const float*>(row) + 4 * (sub + k * LANES);
+      v[k] = make_float4(__ldcs(f), __ldcs(f + 1), __ldcs(f + 2), __ldcs(f + 3));
+    }
+  } else {  // of 8
 #pragma unroll
     for (int k = 0; k < VPL; ++k) {
       const float2 a = __ldcs(row + 2 * (sub + k * LANES)), b = __ldcs(row + 2 * (sub + k * LANES) + 1);
@@ -163,10 +169,18 @@ __device__ __forceinline__ RowSum row_sum(const float2* __restrict__ row, int su
 }
 // complex128: two FP64 FMAs an element, nothing else on the FP64 units but the lanes' sums
 template <int VPL, int LANES>
-__device__ __forceinline__ double row_sum(const double2* __restrict__ row, int sub, bool) {
+__device__ __forceinline__ double row_sum(const double2* __restrict__ row, int sub, int bytes) {
   double2 v[VPL];
+  if (bytes == 16) {
 #pragma unroll
-  for (int k = 0; k < VPL; ++k) v[k] = __ldcs(row + sub + k * LANES);
+    for (int k = 0; k < VPL; ++k) v[k] = __ldcs(row + sub + k * LANES);
+  } else {  // a state on a boundary of 8 bytes
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) {
+      const double* f = reinterpret_cast<const double*>(row + sub + k * LANES);
+      v[k] = make_double2(__ldcs(f), __ldcs(f + 1));
+    }
+  }
   double acc = 0.0;
 #pragma unroll
   for (int k = 0; k < VPL; ++k) acc = fma(v[k].x, v[k].x, fma(v[k].y, v[k].y, acc));
@@ -183,7 +197,7 @@ __device__ __forceinline__ double unpack(double v) { return v; }
 template <typename C, int LOGC>
 __global__ void __launch_bounds__(256, kBlocksPerSM) static_partials_kernel(const C* __restrict__ X, double* __restrict__ probs,
                                                               qpe::Partial* __restrict__ parts, int64_t pieces,
-                                                              int logd, bool vec16) {
+                                                              int logd, int bytes) {
   constexpr int EPV = 16 / (int)sizeof(C);          // elements per 16-byte load
   constexpr int VECS = (1 << LOGC) / EPV;           // loads per piece
   // 64 bytes and more a lane where the row has them, and rows of 16 columns and
@@ -193,7 +207,7 @@ __global__ void __launch_bounds__(256, kBlocksPerSM) static_partials_kernel(cons
   static_assert(LANES >= 1 && LANES <= 32 && VPL * LANES == VECS, "a piece is one warp's loads at most");
   static_assert(sizeof(C) == 16 || VPL <= 4, "the FP32 anchors hold 16 squares a lane");
   constexpr int RPS = 32 / LANES;                   // pieces per warp step
-  using V = decltype(row_sum<VPL, LANES>(static_cast<const C*>(nullptr), 0, true));
+  using V = decltype(row_sum<VPL, LANES>(static_cast<const C*>(nullptr), 0, 16));
   __shared__ V vals[256];
   __shared__ double dv[256];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -208,7 +222,7 @@ __global__ void __launch_bounds__(256, kBlocksPerSM) static_partials_kernel(cons
       const int q = warp * 32 + s + lane / LANES;
       const int64_t piece = base + q < pieces ? base + q : pieces - 1;  // past the end: the last piece again, unused
       const C* p = X + (piece << LOGC);
-      const V v = row_sum<VPL, LANES>(p, lane % LANES, vec16);
+      const V v = row_sum<VPL, LANES>(p, lane % LANES, bytes);
       if (lane % LANES == 0) vals[q] = v;
     }
     __syncwarp();  // a warp reads back only its own pieces
@@ -275,12 +289,13 @@ __global__ void __launch_bounds__(256) static_finish_kernel(const qpe::Partial* 
 template <typename C>
 int launch_partials(const C* X, double* probs, qpe::Partial* parts, int nmat, int nmeas, cudaStream_t s) {
   const int logc = nmat < 8 ? nmat : 8;
-  const bool vec16 = reinterpret_cast<uintptr_t>(X) % 16 == 0;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(X);
+  const int bytes = at % 16 == 0 ? 16 : at % 8 == 0 ? 8 : 4;  // the widest loads X allows
   const int64_t pieces = int64_t(1) << (nmeas + nmat - logc);
   const int64_t tiles = (pieces + 255) / 256;
   const int blocks = (int)(tiles < kMaxBlocks ? tiles : kMaxBlocks);
 #define QPE_PARTIALS(LC) \
-  case LC: static_partials_kernel<C, LC><<<blocks, 256, 0, s>>>(X, probs, parts, pieces, nmat, vec16); break;
+  case LC: static_partials_kernel<C, LC><<<blocks, 256, 0, s>>>(X, probs, parts, pieces, nmat, bytes); break;
   switch (logc) {
     QPE_PARTIALS(1)
     QPE_PARTIALS(2)
@@ -289,7 +304,7 @@ int launch_partials(const C* X, double* probs, qpe::Partial* parts, int nmat, in
     QPE_PARTIALS(5)
     QPE_PARTIALS(6)
     QPE_PARTIALS(7)
-    default: static_partials_kernel<C, 8><<<blocks, 256, 0, s>>>(X, probs, parts, pieces, nmat, vec16); break;
+    default: static_partials_kernel<C, 8><<<blocks, 256, 0, s>>>(X, probs, parts, pieces, nmat, bytes); break;
   }
 #undef QPE_PARTIALS
   return blocks;
@@ -302,6 +317,10 @@ extern "C" qpe_status qpe_readout_static(const void* final_state, int32_t nmat, 
   if (!final_state || !probs || !readout) return QPE_ERR_ARG;
   if (nmat < 1 || nmat > 12 || nmeas < 1 || nmeas > 30) return QPE_ERR_ARG;
   if (prec < QPE_FP64 || prec > QPE_C64_TF32X3) return QPE_ERR_ARG;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(final_state);
+  if (at % (prec == QPE_FP64 ? 8 : 4) || reinterpret_cast<uintptr_t>(probs) % 8 ||
+      reinterpret_cast<uintptr_t>(readout) % 8)
+    return QPE_ERR_ARG;
   if (nmeas > kMaxNmeas) return QPE_ERR_WORKSPACE;
   qpe::Partial* scratch = nullptr;
   cudaError_t e = scratch_address(&scratch);
