@@ -53,7 +53,8 @@ def peaks():
 # the sources that make up each recorded kernel (its translation unit and the
 # headers it includes); a traffic record holds while their code is unchanged
 KERNEL_SOURCES = {
-    "level_oz_top_c5_fp64": ["paper_2507_17175_gb300/csrc/qpe_oztop.cu", "paper_2507_17175_gb300/csrc/qpe_internal.cuh",
+    "level_oz_top_c5_fp64": ["paper_2507_17175_gb300/csrc/qpe_oztop.cu", "paper_2507_17175_gb300/csrc/qpe_fixed.cuh",
+                             "paper_2507_17175_gb300/csrc/qpe_internal.cuh",
                              "paper_2507_17175_gb300/csrc/qpe_tcgen05.cuh", "include/qpe.h"],
 }
 
@@ -478,8 +479,8 @@ def bench_ours(args, rank, world, local_rank):
         "config": {"workload": WORKLOAD, "nmat": inst.nmat, "nmeas": inst.nmeas,
                    "precision": "complex128 state, FP64-accurate: every level of >= 128 pencils as exact integer "
                                 "digit products on the tensor cores (7 x 8-bit digits, Ozaki scheme) with the "
-                                "twiddles and the 8-point DFT in 64-bit fixed point; squaring chain, the deepest "
-                                "levels, |X|^2 and readout in FP64" if top_on_tc else
+                                "twiddles, the 8-point DFT and the sums of |X|^2 in 64-bit fixed point; squaring "
+                                "chain, the deepest levels and readout in FP64" if top_on_tc else
                                 "complex128 state, FP64 arithmetic everywhere (the paper's)",
                    "schedule": f"fused levels ({levels} levels, top level 2^{r_top}-point DFT"
                                f"{' on the tensor cores' if top_on_tc else ''})",

@@ -130,9 +130,9 @@ typedef enum {
                                  /* nmat = 4 the fused schedule's 8-point     */
                                  /* levels of >= 128 pencils, the top level   */
                                  /* included (QPE_INFO_TC_TOP_LEVEL tells;    */
-                                 /* twiddles and DFT in 64-bit fixed point,   */
-                                 /* |X|^2 and readout in FP64; single-        */
-                                 /* instance and sharded plans); with         */
+                                 /* twiddles, DFT and the sums of |X|^2 in    */
+                                 /* 64-bit fixed point, readout in FP64;      */
+                                 /* single-instance and sharded plans); with  */
                                  /* nmat >= 8 the plain schedule's doubling   */
                                  /* levels of >= 128 rows (single-instance,   */
                                  /* sharded and batched plans: one grouped    */

@@ -1070,7 +1070,8 @@ qpe_status qpe_plan_shard(const qpe_plan_desc* desc, int32_t rank, int32_t world
     if (desc->nmeas < 2 * sh || (desc->flags & QPE_FLAG_KEEP_STATE)) return QPE_ERR_UNSUPPORTED;
   } else {
     // the fused form partitions the outcomes; the top level must have at
-    // least `world` pencils
+    // least `world` pencils, of the widest levels: the balanced ones that a plan
+    // of at most 256 outcomes gets have at least as many
     const std::vector<qpe::Level> lv = qpe::make_levels(desc->nmeas, desc->nmat, elem_size(desc->prec), false);
     if (lv.empty() || lv[0].logna < sh) return QPE_ERR_UNSUPPORTED;
   }

@@ -1126,8 +1126,10 @@ bool level_sharded(const Instance& in, int li) {
 // Levels of r <= rmax bits, the top one first. At most 256 outcomes are a matter of
 // latency: a level of five bits is one pencil or two whose 32-point FP64 DFTs and
 // five-factor table rows run on a few lanes of one SM, so `balanced` splits them into
-// equal levels of at most four bits (Nmat 2, Nmeas 6 FP64: the call 132.6 -> 81.4 us,
-// one read-back copy less included; the five-bit top level alone took 61).
+// equal levels of at most four bits. Device time of a run, widest levels and balanced, us:
+// FP64 Nmat 2 with 5 / 6 / 7 / 8 bits 81.6 / 92.3 / 93.7 / 97.5 and 43.9 / 46.9 / 55.2 / 60.0; Nmat 1 77 .. 90
+// and 38 .. 53; complex64 Nmat 1 .. 3 with 6 .. 8 bits 30 .. 36 and 26 .. 35, with 5 bits 24.5 .. 27.3 and
+// 24.5 .. 27.8. Above 8 bits the split is the widest one (not tried otherwise).
 std::vector<Level> make_levels(int nmeas, int logd, size_t esize, bool balanced) {
   int rmax = level_max_bits(logd, esize, kLevelSmemCap);
   if (balanced && nmeas <= 8 && rmax > 4) {

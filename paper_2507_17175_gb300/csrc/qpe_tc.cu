@@ -840,8 +840,8 @@ __device__ __forceinline__ bool oz_move_a(uint32_t tmem, uint32_t aset, int q, i
 }
 
 // One output's sum over the weights in 96 bits: sum_w acc_w 2^(8 (6 - w)) (below
-// 2^76 for K <= 8192); three registers, so that a drain thread's 32 columns and 16
-// accumulators in flight fit 128.
+// 2^76 for K <= 8192) in three registers. A drain thread's 32 columns take 96 of its 128
+// and a few of them spill; the two int64 sums of before took 128.
 struct Oz96 {
   uint32_t w0 = 0, w1 = 0, w2 = 0;
   template <int W>
