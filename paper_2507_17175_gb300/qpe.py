@@ -284,36 +284,38 @@ def _ptr(x):
     raise TypeError(f"unsupported buffer type {type(x)}")
 
 
-def _other_current(stream, device):
-    """The current stream where it is another one than ``stream``, else None.
+def _other_current(plan):
+    """The current stream where it is another one than the plan's, else None.
     None too while it is being captured: an event of a capture cannot order work
-    outside of it, and waiting for one would draw ``stream`` into the capture."""
+    outside of it, and waiting for one would draw the plan's stream into the capture."""
     import torch
-    current = torch.cuda.current_stream(device)
-    if stream.cuda_stream == current.cuda_stream or torch.cuda.is_current_stream_capturing():
+    current = torch.cuda.current_stream(plan._device_index)
+    if plan.stream.cuda_stream == current.cuda_stream or torch.cuda.is_current_stream_capturing():
         return None
     return current
 
 
-def _order_after_current(stream, device, *tensors):
-    """What is enqueued on ``stream`` from here on waits for the current stream:
+def _order_after_current(plan, *tensors):
+    """What is enqueued on the plan's stream from here on waits for the current stream:
     a caller's tensors are written there, and torch hands out memory whose last
-    user there may still be running. ``tensors``: read or written on ``stream``
-    after the call returns; torch keeps their memory until ``stream`` is past that,
+    user there may still be running. ``tensors``: read or written on the plan's stream
+    after the call returns; torch keeps their memory until that stream is past that,
     however early they are dropped."""
-    current = _other_current(stream, device)
+    current = _other_current(plan)
     if current is not None:
-        stream.wait_stream(current)
+        plan._order.record(current)
+        plan.stream.wait_event(plan._order)
         for t in tensors:
             if getattr(t, "is_cuda", False):
-                t.record_stream(stream)
+                t.record_stream(plan.stream)
 
 
-def _order_current_after(stream, device):
-    """What the current stream is given from here on waits for ``stream``."""
-    current = _other_current(stream, device)
+def _order_current_after(plan):
+    """What the current stream is given from here on waits for the plan's."""
+    current = _other_current(plan)
     if current is not None:
-        current.wait_stream(stream)
+        plan._order.record(plan.stream)
+        current.wait_event(plan._order)
 
 
 class Plan:
@@ -342,7 +344,9 @@ class Plan:
         if workspace is None:
             workspace = torch.empty(self.ws_bytes, dtype=torch.uint8, device=self.device)
         self.workspace = workspace
-        _order_after_current(self.stream, self.device, workspace)
+        self._device_index = torch.cuda.current_device() if self.device.index is None else self.device.index
+        self._order = torch.cuda.Event()  # one event, recorded again for each wait
+        _order_after_current(self, workspace)
         self._check(_lib.qpe_bind(self._h, workspace.data_ptr(), self.ws_bytes, self.stream.cuda_stream), "qpe_bind")
 
     def _check(self, st: int, what: str):
@@ -373,7 +377,7 @@ class Plan:
         if du != dp:
             raise ValueError("U and psi must both be host or both be device buffers")
         if du:
-            _order_after_current(self.stream, self.device, U, psi)
+            _order_after_current(self, U, psi)
         self._keep = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, self.nmat, self.nmeas, du), "qpe_load")
 
@@ -404,7 +408,7 @@ class Plan:
             out = np.empty(self.N, dtype=np.float64)
         ptr, dev = (0, 0) if out is None else _ptr(out)
         if dev:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self)
         self._check(_lib.qpe_probs(self._h, instance, ptr or None, ctypes.byref(am), ctypes.byref(pa),
                                    ctypes.byref(pm), dev), "qpe_probs")
         return out, am.value, pa.value, pm.value
@@ -414,10 +418,10 @@ class Plan:
             out = np.empty((self.N, self.d), dtype=self.state_dtype)
         ptr, dev = _ptr(out)
         if dev:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self)
         self._check(_lib.qpe_state(self._h, instance, ptr, dev), "qpe_state")
         if dev:  # enqueued only: what the current stream does with it comes after
-            _order_current_after(self.stream, self.device)
+            _order_current_after(self)
         return out
 
     def load_state(self, S, instance: int = 0):
@@ -425,7 +429,7 @@ class Plan:
             S = np.ascontiguousarray(S, dtype=self.state_dtype)
         ptr, dev = _ptr(S)
         if dev:
-            _order_after_current(self.stream, self.device, S)
+            _order_after_current(self, S)
         self._keep_state = S
         self._check(_lib.qpe_load_state(self._h, instance, ptr, dev), "qpe_load_state")
 
@@ -577,7 +581,7 @@ class BatchedPlan(Plan):
         pu, du = _ptr(U)
         pp, dp = _ptr(psi)
         if du:
-            _order_after_current(self.stream, self.device, U, psi)
+            _order_after_current(self, U, psi)
         self._keep_inputs[instance] = (U, psi)
         self._check(_lib.qpe_load(self._h, instance, pu, pp, nmat, nmeas, du), "qpe_load")
 
@@ -590,7 +594,7 @@ class BatchedPlan(Plan):
             out = np.empty(1 << nmeas, dtype=np.float64)
         ptr, dev = (0, 0) if out is None else _ptr(out)
         if dev:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self)
         self._check(_lib.qpe_probs(self._h, instance, ptr or None, ctypes.byref(am), ctypes.byref(pa),
                                    ctypes.byref(pm), dev), "qpe_probs")
         return out, am.value, pa.value, pm.value
@@ -601,8 +605,8 @@ class BatchedPlan(Plan):
             out = np.empty((1 << nmeas, 1 << nmat), dtype=self.state_dtype)
         ptr, dev = _ptr(out)
         if dev:
-            _order_after_current(self.stream, self.device)
+            _order_after_current(self)
         self._check(_lib.qpe_state(self._h, instance, ptr, dev), "qpe_state")
         if dev:  # enqueued only: what the current stream does with it comes after
-            _order_current_after(self.stream, self.device)
+            _order_current_after(self)
         return out

@@ -15,8 +15,13 @@ class _Stream:
     def __init__(self, handle, log):
         self.cuda_stream, self.log = handle, log
 
-    def wait_stream(self, other):
-        self.log.append(("wait", self.cuda_stream, other.cuda_stream))
+    def wait_event(self, event):
+        self.log.append(("wait", self.cuda_stream, event.recorded))
+
+
+class _Event:
+    def record(self, stream):
+        self.recorded = stream.cuda_stream
 
 
 class _Tensor(torch.Tensor):
@@ -52,6 +57,8 @@ def recorded(monkeypatch):
     monkeypatch.setattr(qpe, "_lib", _Lib(log))
     monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: _Stream(CURRENT, log))
     monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: capturing[0])
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "Event", _Event)
 
     def make(cls=qpe.Plan, handle=OWN):
         p = object.__new__(cls)
@@ -59,6 +66,7 @@ def recorded(monkeypatch):
         p.nmat, p.nmeas, p.d, p.N = 1, 2, 2, 4
         p.shapes, p._keep_inputs = [(1, 2)], {}
         p.stream, p.device = _Stream(handle, log), torch.device("cuda")
+        p._device_index, p._order = 0, _Event()
         return p
     yield make, log, capturing
     log.clear()
