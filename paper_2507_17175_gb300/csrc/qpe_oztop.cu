@@ -37,7 +37,7 @@
 // bits). The fixed point's truncations are a few units, 2^-56 of the pencil's
 // bound |T| < 2^(tau + sigma + 5), below the contraction's own error. The sums
 // over the warps and the readout run in FP64. Top level at Nmeas 24: 4.0 ms with
-// its lower levels before the MMA warp ran converged, 3.2 so (2.48 ms alone).
+// its lower levels before the MMA warp ran converged, 3.3 so (2.52 ms alone).
 //
 // Roles (640 threads, one CTA per SM, persistent over the tiles):
 //   warps 0-2   producers: Z rows -> digit tiles (shared memory, 128-byte
